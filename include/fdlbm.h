@@ -120,10 +120,13 @@ typedef struct {
     double rho0;              /* reference density; FP32 storage keeps f~_i - w_i rho0 */
     int precision;            /* FDLBM_FP64 or FDLBM_FP32_DEV */
     int has_force;            /* 1: reserve a body-acceleration field (fdlbm_set_force), Eq. 3.12 */
-    int path;                 /* FDLBM_PATH_AUTO: the fused kernel for both schemes on periodic
-                                 grids and on walled grids in FP32; the staged kernels for
-                                 walled grids in FP64 (bound by the FP64 units, where the
-                                 sweep's recomputed halo costs more than the extra traffic) */
+    int path;                 /* FDLBM_PATH_AUTO: the fused path for both schemes on periodic
+                                 grids and on walled grids in FP32; the staged path for
+                                 walled grids in FP64.  T2S2-FDLBM1 takes the split step (two
+                                 launches per step and one more per call, one node per
+                                 thread, no halo recomputed) on the staged path, and in FP64
+                                 on either one unless rows_per_cta or variant is set: FP64
+                                 is bound by the FP64 units */
     int rows_per_cta;         /* fused kernel tile height; 0 = automatic */
     int variant;              /* FDLBM_VARIANT_*; WARP where it does not apply -> EUNSUPPORTED */
     int scheme;               /* FDLBM_SCHEME_T2S2_1 (default) or FDLBM_SCHEME_T2S2_2 */
@@ -223,7 +226,8 @@ double fdlbm_dt(fdlbm_t h);              /* the dt of Eq. 3.1 used by the handle
 double fdlbm_tau(fdlbm_t h);             /* nu / cs^2 */
 long long fdlbm_steps_done(fdlbm_t h);   /* steps enqueued since creation */
 int fdlbm_path(fdlbm_t h);               /* FDLBM_PATH_FUSED or FDLBM_PATH_STAGED */
-int fdlbm_kernels_per_step(fdlbm_t h);   /* kernel launches fdlbm_step makes per step */
+int fdlbm_kernels_per_step(fdlbm_t h);   /* kernel launches fdlbm_step makes per step (the split
+                                            step makes one more per call or graph replay) */
 /* The tiles of the warp-tile kernel's step on a grid (FDLBM_VARIANT_WARP), for
  * the tile height `rows` (> 0) and `scheme` (FDLBM_SCHEME_*): first the
  * interior windows in launch order, then, on a walled grid, the frame tiles,

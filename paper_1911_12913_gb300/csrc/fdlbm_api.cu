@@ -76,11 +76,11 @@ bool fused_ok(const fdlbm_grid *g) { return g->nx >= 4 && g->ny >= 4; }
 
 bool walled(const fdlbm_grid *g) { return g->bc_x == FDLBM_WALL || g->bc_y == FDLBM_WALL; }
 
-// The automatic choice takes the fused sweep for T2S2-FDLBM1, except on walled
-// grids in FP64: there the work is bound by the FP64 units, and the halo rows
-// the sweep recomputes on small walled grids cost more than the staged
-// kernels' extra traffic (257^2 cavity: 198 against 81 us per step on GB300).
-// Both schemes have fused sweeps, for periodic and walled grids.
+// The automatic choice is the fused path, except on walled grids in FP64: there
+// the work is bound by the FP64 units, and the halo rows the sweeps recompute
+// cost more than the extra traffic of stages that meet in scratch fields
+// (T2S2-FDLBM1 in FP64 takes the split step on either path: use_split).  Both
+// schemes have fused sweeps, for periodic and walled grids.
 int choose_path(const fdlbm_grid *g, const fdlbm_opts *o)
 {
     const bool can_fuse = fused_ok(g);
@@ -88,6 +88,28 @@ int choose_path(const fdlbm_grid *g, const fdlbm_opts *o)
     if (o->path == FDLBM_PATH_FUSED) return can_fuse ? FDLBM_PATH_FUSED : -1;
     if (walled(g) && o->precision == FDLBM_FP64) return FDLBM_PATH_STAGED;
     return can_fuse ? FDLBM_PATH_FUSED : FDLBM_PATH_STAGED;
+}
+
+// T2S2-FDLBM1 in two launches per step (step_split.cu) where the staged path
+// is taken, and for FP64 grids unless a tile height or a kernel is asked for.
+// FP64 is bound by the FP64 units, and the split step does no node's work
+// twice (us per step on GB300, sweep or staged kernels -> split: 64^2 periodic
+// 59.6 -> 11.6, 257^2 cavity 81 -> 35, 1024^2 periodic 718 -> 431); in FP32 the
+// sweeps move a third of its bytes (2048^2: 70 against 205).
+bool use_split(const fdlbm_opts *o, int path)
+{
+    if (o->scheme != FDLBM_SCHEME_T2S2_1) return false;
+    if (path == FDLBM_PATH_STAGED) return true;
+    return o->precision == FDLBM_FP64 && o->path == FDLBM_PATH_AUTO && o->variant == FDLBM_VARIANT_AUTO &&
+           o->rows_per_cta == 0;
+}
+
+// Scratch fields a handle needs (see make_layout).
+int scratch_fields(const fdlbm_grid *g, const fdlbm_opts *o, int path, bool force_staged)
+{
+    if (force_staged || path == FDLBM_PATH_STAGED || o->adjoint) return 3;
+    if (use_split(o, path)) return walled(g) ? 2 : 1;
+    return 0;
 }
 
 // Rows per CTA of the fused kernel.  Each CTA recomputes 8 halo rows, so tall
@@ -152,12 +174,28 @@ StepArgs<R> step_args(fdlbm_ctx *h)
     a.stc = make_stencil<R>(0.0);
     a.rows = h->rows;
     a.err = reinterpret_cast<int *>(h->ws + h->lay.err);
-    if (h->path == FDLBM_PATH_STAGED || h->adjoint) {
+    if (h->lay.S) {
         a.P = reinterpret_cast<R *>(h->ws + h->lay.P);
         a.Q = reinterpret_cast<R *>(h->ws + h->lay.Q);
         a.S = reinterpret_cast<R *>(h->ws + h->lay.S);
     }
     return a;
+}
+
+template <class R>
+cudaError_t launch_split_steps(fdlbm_ctx *h, int n, cudaStream_t s)
+{
+    const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
+    R *q0 = reinterpret_cast<R *>(h->ws + h->lay.Q);
+    R *q1 = walls ? reinterpret_cast<R *>(h->ws + h->lay.P) : q0;
+    return launch_split<R>(step_args<R>(h), q0, q1, reinterpret_cast<const R *>(h->ws + h->lay.split), n, s);
+}
+
+// n steps of the split kernels (the state stays in state[cur]), on stream s.
+cudaError_t launch_split_steps(fdlbm_ctx *h, int n, cudaStream_t s)
+{
+    return h->precision == FDLBM_FP32_DEV ? launch_split_steps<float>(h, n, s)
+                                          : launch_split_steps<double>(h, n, s);
 }
 
 // One step of whichever kernel the handle uses, reading state[cur], on stream s.
@@ -181,6 +219,12 @@ cudaError_t launch_step(fdlbm_ctx *h, cudaStream_t s)
 
 fdlbm_status step_direct(fdlbm_ctx *h, int n)
 {
+    if (h->split) {
+        cudaError_t e = launch_split_steps(h, n, h->stream);
+        if (e != cudaSuccess) return cuda_fail(h, e, "step");
+        h->steps += n;
+        return FDLBM_OK;
+    }
     for (int k = 0; k < n; ++k) {
         cudaError_t e = launch_step(h, h->stream);
         if (e != cudaSuccess) return cuda_fail(h, e, "step");
@@ -212,7 +256,8 @@ fdlbm_status capture_step_graph(fdlbm_ctx *h)
     cudaError_t el = cudaSuccess;
     const int cur0 = h->cur;
     if (e == cudaSuccess) {
-        for (int k = 0; k < h->graph_steps && el == cudaSuccess; ++k) {
+        if (h->split) el = launch_split_steps(h, h->graph_steps, cs);
+        for (int k = 0; k < h->graph_steps && el == cudaSuccess && !h->split; ++k) {
             h->cur = k & 1;
             el = launch_step(h, cs);
         }
@@ -384,7 +429,7 @@ namespace fdlbm {
 
 size_t real_size(int precision) { return precision == FDLBM_FP32_DEV ? 4 : 8; }
 
-Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, bool staged)
+Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, int scratch, bool split)
 {
     Layout L{};
     const size_t rs = real_size(precision);
@@ -402,11 +447,10 @@ Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, bool
     L.mxd = take(nx * sizeof(double));
     L.myd = take(ny * sizeof(double));
     L.force = has_force ? take(2 * plane * rs) : 0;
-    if (staged) {
-        L.P = take(9 * plane * rs);
-        L.Q = take(9 * plane * rs);
-        L.S = take(9 * plane * rs);
-    }
+    if (scratch > 0) L.Q = take(9 * plane * rs);
+    if (scratch > 1) L.P = take(9 * plane * rs);
+    if (scratch > 2) L.S = take(9 * plane * rs);
+    if (split) L.split = take(split_table_bytes(nx, ny, rs));
     L.uprev = take(2 * (size_t)nx * ny * sizeof(double));
     L.nblocks_red = kRedBlocks;
     L.partials = take((size_t)kRedBlocks * 3 * sizeof(double));
@@ -499,11 +543,26 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->stream = static_cast<cudaStream_t>(o.stream);
     h->adjoint = o.adjoint != 0;
     h->graph_steps = o.graph_steps > 0 ? o.graph_steps + (o.graph_steps & 1) : 0;
+    h->split = !force_staged && use_split(&o, path);
     h->lay = make_layout(h->nx, h->ny, h->pitch, h->precision, h->has_force,
-                         path == FDLBM_PATH_STAGED || h->adjoint);
+                         scratch_fields(g, &o, path, force_staged), h->split);
     cudaGetDevice(&h->device);
     *out = h;
     return FDLBM_OK;
+}
+
+template <class R>
+static cudaError_t upload_split_tables_t(fdlbm_ctx *h, const std::vector<double> &mx, const std::vector<double> &my)
+{
+    const std::vector<R> t = make_split_tables<R>(mx, my, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, h->beta,
+                                                  h->A * h->dt, h->dt);
+    return cudaMemcpy(h->ws + h->lay.split, t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice);
+}
+
+static cudaError_t upload_split_tables(fdlbm_ctx *h, const std::vector<double> &mx, const std::vector<double> &my)
+{
+    return h->precision == FDLBM_FP32_DEV ? upload_split_tables_t<float>(h, mx, my)
+                                          : upload_split_tables_t<double>(h, mx, my);
 }
 
 // Zero the state (fluid at rest) and the force, clear the error flag, upload
@@ -534,6 +593,7 @@ fdlbm_status handle_upload(fdlbm_ctx *h, const std::vector<double> &mx, const st
         e = cudaMemcpy(h->ws + h->lay.mxd, mx.data(), mx.size() * 8, cudaMemcpyHostToDevice);
     if (e == cudaSuccess)
         e = cudaMemcpy(h->ws + h->lay.myd, my.data(), my.size() * 8, cudaMemcpyHostToDevice);
+    if (e == cudaSuccess && h->split) e = upload_split_tables(h, mx, my);
     if (e == cudaSuccess) e = cudaStreamSynchronize(h->stream);
     return e == cudaSuccess ? FDLBM_OK : FDLBM_ECUDA;
 }
@@ -577,7 +637,7 @@ size_t fdlbm_workspace_bytes(const fdlbm_grid *g, const fdlbm_opts *opts)
     const int path = choose_path(g, &o);
     if (path < 0) return 0;
     return make_layout(g->nx, g->ny, pitch_of(g->nx), o.precision, o.has_force,
-                       path == FDLBM_PATH_STAGED || o.adjoint)
+                       scratch_fields(g, &o, path, false), use_split(&o, path))
         .total;
 }
 
@@ -813,6 +873,7 @@ int fdlbm_kernels_per_step(fdlbm_t h)
 {
     if (!h) return -1;
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
+    if (h->split) return 2;  // and one more per fdlbm_step call (or graph replay)
     if (h->path == FDLBM_PATH_FUSED) {
         // a walled grid on the warp-tile kernel: the frame's launch and the interior's
         if (h->precision == FDLBM_FP32_DEV && h->variant == FDLBM_VARIANT_WARP && walls) {
@@ -933,11 +994,13 @@ const char *fdlbm_describe(fdlbm_t h)
         return h->desc.c_str();
     }
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
-    const char *kern = h->path == FDLBM_PATH_STAGED        ? "staged"
+    const char *kern = h->split                            ? "split"
+                       : h->path == FDLBM_PATH_STAGED      ? "staged"
                        : h->variant == FDLBM_VARIANT_WARP   ? "fused-warp"
                        : walls                              ? "fused-walls"
                                                             : "fused";
-    h->desc = std::string(kern) + " " + prec + " rows=" + std::to_string(h->rows);
+    h->desc = std::string(kern) + " " + prec;
+    if (!h->split) h->desc += " rows=" + std::to_string(h->rows);
     if (walls && h->path == FDLBM_PATH_FUSED && h->variant == FDLBM_VARIANT_WARP) h->desc += " walls";
     if (h->graph_steps) h->desc += " graph_steps=" + std::to_string(h->graph_steps);
     if (h->incomp) h->desc += " incompressible";

@@ -56,7 +56,7 @@ struct WarpMaps {
 };
 
 struct Layout {
-    size_t state[2], mx, my, mxd, myd, force, P, Q, S, uprev, partials, red, err, staging;
+    size_t state[2], mx, my, mxd, myd, force, P, Q, S, split, uprev, partials, red, err, staging;
     size_t staging_elems, total;
     int nblocks_red;
 };
@@ -77,6 +77,7 @@ struct fdlbm_ctx {
     int variant = FDLBM_VARIANT_SCALAR;  // fused kernel actually used
     bool in_batch = false;               // owned by a batch: stepped by fdlbm_batch_step
     bool adjoint = false;                // scratch for the adjoint step reserved
+    bool split = false;                  // two launches per step (step_split.cu), in place
     int graph_steps = 0;                 // steps per replayed CUDA graph (even), 0 = none
     fdlbm::WarpMaps wmaps{};             // tensor maps of the warp-tile kernel
     cudaGraph_t graph = nullptr;
@@ -105,7 +106,9 @@ fdlbm_status handle_upload(fdlbm_ctx *h, const std::vector<double> &mx,
                            const std::vector<double> &my);
 template <class R>
 StepArgs<R> handle_step_args(fdlbm_ctx *h);
-Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, bool staged);
+// Scratch fields of a handle: all three (staged kernels, adjoint), or the f~+
+// buffers of the split step (two on walled grids), and the split step's tables.
+Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, int scratch, bool split);
 
 // step_fused.cu
 template <class R>
@@ -176,6 +179,14 @@ template <class R>
 cudaError_t launch_batched_fused(const BatchTables &t, int parity, int blk_off, int nblocks,
                                  cudaStream_t s);
 int fused_tile_width_walls();
+// step_split.cu (two launches per step, one node per thread; the state in
+// s.gin is advanced in place, s.gout is scratch)
+size_t split_table_bytes(int nx, int ny, size_t real_size);
+template <class R>
+std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
+                                 double beta, double h, double dt);
+template <class R>
+cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream);
 // step_staged.cu
 template <class R>
 cudaError_t launch_staged(const StepArgs<R> &a, cudaStream_t s);

@@ -1,0 +1,577 @@
+// The T2S2-FDLBM1 step in two launches per step, one node per thread, for any
+// boundary combination: each quantity of Sec. 2D is formed once per node, with
+// no halo recomputed.
+//
+//   k_split_prepare  first launch of a call: f~ -> P = fbar^{+,h} (Eqs. 2.19,
+//                    2.34), written over f~, and Q = f~+ (Eq. 2.20)
+//   k_split_star     P -> S = f* (Eqs. 2.32-2.35; Eq. 3.10 at wall nodes)
+//   k_split_update   Q, S -> f~ of the next step (Eq. 2.23; Eq. 3.10 at wall
+//                    nodes) and, in registers, its P and Q; the last step of a
+//                    call stores f~ instead
+//
+// A wall node's thread works at its nearest interior node x_j and extrapolates
+// from there, so that walls need no launch of their own; it reads Q of another
+// node, so on walled grids Q alternates between two buffers.
+//
+// The difference weights come from tables with the metric, the time step and
+// the sign folded in (make_split_tables): one multiply-add per tap, and next to
+// a wall, where the second-order upwind tap would leave the domain, the entry
+// of that sign holds the central difference.
+//
+// What bounds it.  FP64: the FP64 units, 227 FP64 instructions per node (prepare
+// 79, star 104, update 44): 1024^2 periodic 431 us per step, 0.87 of the rate at
+// which a warp's FP64 instruction takes 64 cycles of its scheduler; the 576
+// bytes per node that pass between the launches are hidden behind them.  The
+// sweep it replaced there recomputed 8 halo rows and columns per tile and spent
+// 281 instructions per node: 718 us.  Small grids wait for launches and for one
+// warp's chain of instructions: 64^2 11.6 us per step (sweep 59.6), 257^2 cavity
+// 35.1 (five staged launches with a thread per wall node 81).
+#include <algorithm>
+#include <cmath>
+#include <vector>
+
+#include "internal.h"
+#include "walls_nodes.cuh"
+
+namespace fdlbm {
+namespace {
+
+// Threads per block.  FP64: one warp.  A warp's FP64 instruction holds its
+// scheduler's FP64 unit for 64 cycles, so a launch lasts as long as the
+// scheduler with the most warps; single warps spread most evenly (257^2 cavity:
+// 35.1 us per step, 45.5 in blocks of 128, 1024^2: the same either way).
+template <class R>
+constexpr int kThreads = sizeof(R) == 8 ? 32 : 128;
+
+// Wait for the previous launch of the chain (its results are visible after
+// this); let the next one's blocks be scheduled.  The second comes after a
+// warp's arithmetic: at the start of the kernel, the waiting blocks of the next
+// launch took SM slots unevenly (257^2 periodic FP64: 31.4 us per step against
+// 51.6; without the chain attribute 35.2).
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+template <class R>
+struct SplitArgs {
+    R *P, *S;                // [9][ny][pitch]; S: planes 1 to 8 (population 0 does not move)
+    const R *Qin;            // f~+ of this step
+    R *Qout;                 // f~+ of the next step (k_split_update), or f~ (its last launch)
+    const R *force;
+    const R *tx, *ty;        // weight tables of the stage: [n][2][4] (sign +, sign -)
+    int nx, ny, pitch;
+    size_t plane;
+    int wx, wy;
+    int x0, y0, w, h;        // rectangle of the launch: all nodes, or the interior ones
+    int strip, strip_blocks; // strip width (threads run along rows of a strip), blocks per strip
+    int wall_blocks;         // leading blocks that take the wall nodes
+    R wall_u[4][2];
+    Coeffs<R> c;
+    R keep_star, w_star[3], l_star[2];  // (1 - b*)/2, b* w_i, b* c_i of the linear terms
+};
+
+template <class R>
+struct Taps {
+    R m1, c, p1, p2;         // at k + s, k, k - s, k - 2s for velocity sign s
+};
+
+template <class R>
+__device__ __forceinline__ Taps<R> load_taps(const R *t)
+{
+    Taps<R> w;
+    if constexpr (sizeof(R) == 4) {
+        const float4 v = __ldg(reinterpret_cast<const float4 *>(t));
+        w.m1 = v.x;
+        w.c = v.y;
+        w.p1 = v.z;
+        w.p2 = v.w;
+    } else {
+        const double2 u = __ldg(reinterpret_cast<const double2 *>(t));
+        const double2 v = __ldg(reinterpret_cast<const double2 *>(t) + 1);
+        w.m1 = u.x;
+        w.c = u.y;
+        w.p1 = v.x;
+        w.p2 = v.y;
+    }
+    return w;
+}
+
+// A node, its neighbours (wrapped on a periodic axis; on a walled axis clamped,
+// where the weights are zero) and the weights of its differences.
+template <class R, bool WALLS>
+struct Site {
+    int x[5], y[5];          // k - 2 .. k + 2
+    Taps<R> xp, xn, yp, yn;  // weights for the signs of each axis
+
+    __device__ __forceinline__ void set(const SplitArgs<R> &a, int xc, int yc)
+    {
+#pragma unroll
+        for (int d = -2; d <= 2; ++d) {
+            int u = xc + d, v = yc + d;
+            if (WALLS && a.wx) u = min(max(u, 0), a.nx - 1);
+            else u = u < 0 ? u + a.nx : (u >= a.nx ? u - a.nx : u);
+            if (WALLS && a.wy) v = min(max(v, 0), a.ny - 1);
+            else v = v < 0 ? v + a.ny : (v >= a.ny ? v - a.ny : v);
+            x[d + 2] = u;
+            y[d + 2] = v * a.pitch;
+        }
+        xp = load_taps(a.tx + 8 * xc);
+        yp = load_taps(a.ty + 8 * yc);
+        xn = WALLS ? load_taps(a.tx + 8 * xc + 4) : xp;
+        yn = WALLS ? load_taps(a.ty + 8 * yc + 4) : yp;
+    }
+
+    // acc plus the weighted taps of population i of plane f around the node
+    __device__ __forceinline__ R advance(const R *f, int i, R v0, R acc) const
+    {
+        const int r0 = y[2];
+        if constexpr (sizeof(R) == 8) {
+            // FP64: one multiply-add per tap, the centre weights of a diagonal merged
+            if (cx(i) != 0 && cy(i) != 0) acc = fma((cx(i) > 0 ? xp.c : xn.c) + (cy(i) > 0 ? yp.c : yn.c), v0, acc);
+            else if (cx(i) != 0) acc = fma(cx(i) > 0 ? xp.c : xn.c, v0, acc);
+            else acc = fma(cy(i) > 0 ? yp.c : yn.c, v0, acc);
+            if (cx(i) != 0) {
+                const Taps<R> &w = cx(i) > 0 ? xp : xn;
+                const int s = cx(i);
+                acc = fma(w.m1, f[r0 + x[2 + s]], acc);
+                acc = fma(w.p1, f[r0 + x[2 - s]], acc);
+                acc = fma(w.p2, f[r0 + x[2 - 2 * s]], acc);
+            }
+            if (cy(i) != 0) {
+                const Taps<R> &w = cy(i) > 0 ? yp : yn;
+                const int s = cy(i);
+                acc = fma(w.m1, f[y[2 + s] + x[2]], acc);
+                acc = fma(w.p1, f[y[2 - s] + x[2]], acc);
+                acc = fma(w.p2, f[y[2 - 2 * s] + x[2]], acc);
+            }
+            return acc;
+        } else {
+            // FP32: the difference first, so that the sum rounds to acc's size once
+            R d = R(0);
+            if (cx(i) != 0) {
+                const Taps<R> &w = cx(i) > 0 ? xp : xn;
+                const int s = cx(i);
+                d = w.c * v0;
+                d = fma(w.m1, f[r0 + x[2 + s]], d);
+                d = fma(w.p1, f[r0 + x[2 - s]], d);
+                d = fma(w.p2, f[r0 + x[2 - 2 * s]], d);
+            }
+            if (cy(i) != 0) {
+                const Taps<R> &w = cy(i) > 0 ? yp : yn;
+                const int s = cy(i);
+                d = cx(i) != 0 ? fma(w.c, v0, d) : w.c * v0;
+                d = fma(w.m1, f[y[2 + s] + x[2]], d);
+                d = fma(w.p1, f[y[2 - s] + x[2]], d);
+                d = fma(w.p2, f[y[2 - 2 * s] + x[2]], d);
+            }
+            return acc + d;
+        }
+    }
+};
+
+// Node coordinates of this thread.  Wall nodes come first, in blocks of their
+// own (a warp that holds both kinds would run Eq. 3.10 for its interior lanes
+// too); then the rectangle, linear over strips of `strip` columns, so that
+// every warp is full on any width.  False past the end.
+template <class R, bool WALLS>
+__device__ __forceinline__ bool my_node(const SplitArgs<R> &a, int &x, int &y)
+{
+    if (WALLS && blockIdx.x < a.wall_blocks) {
+        const int k = blockIdx.x * blockDim.x + threadIdx.x;
+        const int rows = a.wy ? 2 * a.nx : 0;  // S and N rows, corners included
+        if (k < rows) {
+            x = k < a.nx ? k : k - a.nx;
+            y = k < a.nx ? 0 : a.ny - 1;
+            return true;
+        }
+        const int len = a.wy ? a.ny - 2 : a.ny, m = k - rows;  // W and E columns
+        x = m < len ? 0 : a.nx - 1;
+        y = (m < len ? m : m - len) + (a.wy ? 1 : 0);
+        return a.wx && m < 2 * len;
+    }
+    const int b = blockIdx.x - (WALLS ? a.wall_blocks : 0);
+    const int strip = b / a.strip_blocks;
+    const unsigned k = (b - strip * a.strip_blocks) * blockDim.x + threadIdx.x;
+    const int xs = strip * a.strip;
+    const unsigned w = min(a.strip, a.w - xs);
+    const unsigned row = k / w;
+    x = a.x0 + xs + (int)(k - row * w);
+    y = a.y0 + (int)row;
+    return row < (unsigned)a.h;
+}
+
+// The wall that owns node (x, y) and its interior neighbour x_j along the
+// inward normal (diagonal at corners; the W/E walls own the corners); -1 at an
+// interior node, whose x_j is itself.
+template <class R>
+__device__ __forceinline__ int wall_side(const SplitArgs<R> &a, int x, int y, int &jx, int &jy)
+{
+    jx = a.wx ? min(max(x, 1), a.nx - 2) : x;
+    jy = a.wy ? min(max(y, 1), a.ny - 2) : y;
+    if (jx != x) return x == 0 ? FDLBM_WALL_W : FDLBM_WALL_E;
+    if (jy != y) return y == 0 ? FDLBM_WALL_S : FDLBM_WALL_N;
+    return -1;
+}
+
+template <class R>
+__device__ __forceinline__ void wall_velocity(const SplitArgs<R> &a, int side, R &u, R &v)
+{
+    u = v = R(0);
+#pragma unroll
+    for (int s = 0; s < 4; ++s)
+        if (s == side) {
+            u = a.wall_u[s][0];
+            v = a.wall_u[s][1];
+        }
+}
+
+// Sums and differences of opposite populations, and the moments from them:
+// pairs (1,3), (2,4), (5,7), (6,8).
+template <class R>
+struct Node {
+    R s[4], d[4], drho, jx, jy, inv, base, h45, e[4];
+
+    __device__ __forceinline__ void moments(const R g[9])
+    {
+        const int a[4] = {1, 2, 5, 6}, b[4] = {3, 4, 7, 8};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            s[k] = g[a[k]] + g[b[k]];
+            d[k] = g[a[k]] - g[b[k]];
+        }
+        drho = g[0] + ((s[0] + s[1]) + (s[2] + s[3]));
+        jx = d[0] + (d[2] - d[3]);
+        jy = d[1] + (d[2] + d[3]);
+    }
+    // Eq. 3.2 in pairs: f^eq - w rho0 = w t +- c e with t = drho + (4.5 e^2 -
+    // 1.5 j.j)/rho (see equilibrium_dev_j); t of the rest population is base
+    __device__ __forceinline__ void equilibrium(const Coeffs<R> &c)
+    {
+        inv = node_reciprocal(macro_density(c, drho));
+        const R q = jx * jx + jy * jy;
+        h45 = R(4.5) * inv;
+        base = fma(q, R(-1.5) * inv, drho);
+        e[0] = jx;
+        e[1] = jy;
+        e[2] = jx + jy;
+        e[3] = jy - jx;
+    }
+    __device__ __forceinline__ R t(int k) const { return fma(e[k] * e[k], h45, base); }
+    __device__ __forceinline__ static R w(int k) { return k < 2 ? wq<R>(1) : wq<R>(5); }
+    __device__ __forceinline__ static R lin(int k) { return k < 2 ? LinearCoef<R>::c1 : LinearCoef<R>::c2; }
+};
+
+// P and Q of one node from its f~ (g): g + b (f^eq - g) + c F.
+template <class R, bool FORCE>
+__device__ __forceinline__ void prepare(const SplitArgs<R> &a, const R g[9], R Fx, R Fy, R P[9], R Q[9])
+{
+    const Coeffs<R> &c = a.c;
+    if constexpr (FORCE) {
+        R drho, rho, ux, uy, geq[9], F[9];
+        node_eq<R, true>(c, g, Fx, Fy, c.half_dt, drho, rho, ux, uy, geq);
+        force_terms(c.rho0, geq, ux, uy, Fx, Fy, F, force_dshift(c, drho));
+#pragma unroll
+        for (int i = 0; i < 9; ++i) {
+            const R neq = geq[i] - g[i];
+            P[i] = g[i] + c.b_bar * neq + c.c_bar * F[i];
+            Q[i] = g[i] + c.b_til * neq + c.c_til * F[i];
+        }
+    } else {
+        Node<R> n;
+        n.moments(g);
+        n.equilibrium(c);
+        const R neq0 = fma(wq<R>(0), n.base, -g[0]);
+        P[0] = fma(c.b_bar, neq0, g[0]);
+        Q[0] = fma(c.b_til, neq0, g[0]);
+        const int ia[4] = {1, 2, 5, 6}, ib[4] = {3, 4, 7, 8};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const R sym = fma(n.s[k], R(-0.5), n.w(k) * n.t(k));
+            const R asym = fma(n.d[k], R(-0.5), n.lin(k) * n.e[k]);
+            const R na = sym + asym, nb = sym - asym;
+            P[ia[k]] = fma(c.b_bar, na, g[ia[k]]);
+            P[ib[k]] = fma(c.b_bar, nb, g[ib[k]]);
+            Q[ia[k]] = fma(c.b_til, na, g[ia[k]]);
+            Q[ib[k]] = fma(c.b_til, nb, g[ib[k]]);
+        }
+    }
+}
+
+// f* of populations 1 to 8 (and 0 if REST) from fbar* (gs): gs + b* (f^eq - gs) + c* F.
+template <class R, bool FORCE, bool REST>
+__device__ __forceinline__ void relax_star(const SplitArgs<R> &a, const R gs[9], R Fx, R Fy, R st[9])
+{
+    const Coeffs<R> &c = a.c;
+    if constexpr (FORCE) {
+        R drho, rho, ux, uy, geq[9], F[9];
+        node_eq<R, true>(c, gs, Fx, Fy, c.half_h, drho, rho, ux, uy, geq);
+        force_terms(c.rho0, geq, ux, uy, Fx, Fy, F, force_dshift(c, drho));
+#pragma unroll
+        for (int i = REST ? 0 : 1; i < 9; ++i) st[i] = gs[i] + c.b_star * (geq[i] - gs[i]) + c.c_star * F[i];
+    } else {
+        Node<R> n;
+        n.moments(gs);
+        n.equilibrium(c);
+        if (REST) st[0] = fma(a.w_star[0], n.base, (a.keep_star + a.keep_star) * gs[0]);
+        const int ia[4] = {1, 2, 5, 6}, ib[4] = {3, 4, 7, 8};
+#pragma unroll
+        for (int k = 0; k < 4; ++k) {
+            const R sym = fma(a.keep_star, n.s[k], a.w_star[k < 2 ? 1 : 2] * n.t(k));
+            const R asym = fma(a.keep_star, n.d[k], a.l_star[k < 2 ? 0 : 1] * n.e[k]);
+            st[ia[k]] = sym + asym;
+            st[ib[k]] = sym - asym;
+        }
+    }
+}
+
+template <class R, bool FORCE>
+__device__ __forceinline__ void load_force(const SplitArgs<R> &a, int x, int y, R &Fx, R &Fy)
+{
+    Fx = Fy = R(0);
+    if (FORCE) {
+        const size_t o = (size_t)y * a.pitch + x;
+        Fx = __ldg(a.force + o);
+        Fy = __ldg(a.force + a.plane + o);
+    }
+}
+
+template <class R, bool FORCE>
+__global__ void __launch_bounds__(kThreads<R>) k_split_prepare(const SplitArgs<R> a)
+{
+    int x, y;
+    if (!my_node<R, false>(a, x, y)) return;
+    const size_t o = (size_t)y * a.pitch + x;
+    R g[9], P[9], Q[9], Fx, Fy;
+#pragma unroll
+    for (int i = 0; i < 9; ++i) g[i] = a.P[i * a.plane + o];
+    load_force<R, FORCE>(a, x, y, Fx, Fy);
+    prepare<R, FORCE>(a, g, Fx, Fy, P, Q);
+    chain_next();
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        a.P[i * a.plane + o] = P[i];
+        a.Qout[i * a.plane + o] = Q[i];
+    }
+}
+
+template <class R, bool FORCE, bool WALLS>
+__global__ void __launch_bounds__(kThreads<R>) k_split_star(const SplitArgs<R> a)
+{
+    int x, y;
+    if (!my_node<R, WALLS>(a, x, y)) return;
+    int jx = x, jy = y, side = -1;
+    if (WALLS) side = wall_side(a, x, y, jx, jy);
+    Site<R, WALLS> n;
+    n.set(a, jx, jy);
+    R Fx, Fy;
+    load_force<R, FORCE>(a, jx, jy, Fx, Fy);
+    chain_wait();
+    R gs[9], st[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const R *f = a.P + i * a.plane;
+        const R v0 = f[n.y[2] + n.x[2]];
+        gs[i] = i == 0 ? v0 : n.advance(f, i, v0, v0);
+    }
+    relax_star<R, FORCE, WALLS>(a, gs, Fx, Fy, st);
+    if (WALLS && side >= 0) {  // Eq. 3.10 for f* (no force shift)
+        R u, v, wv[9];
+        wall_velocity(a, side, u, v);
+        nee<R, false>(a.c, st, R(0), R(0), R(0), u, v, wv);
+#pragma unroll
+        for (int i = 1; i < 9; ++i) st[i] = wv[i];
+    }
+    chain_next();
+    const size_t o = (size_t)y * a.pitch + x;
+#pragma unroll
+    for (int i = 1; i < 9; ++i) a.S[i * a.plane + o] = st[i];
+}
+
+template <class R, bool FORCE, bool WALLS, bool LAST>
+__global__ void __launch_bounds__(kThreads<R>) k_split_update(const SplitArgs<R> a)
+{
+    int x, y;
+    if (!my_node<R, WALLS>(a, x, y)) return;
+    int jx = x, jy = y, side = -1;
+    if (WALLS) side = wall_side(a, x, y, jx, jy);
+    Site<R, WALLS> n;
+    n.set(a, jx, jy);
+    chain_wait();
+    R g[9];
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        const int o0 = n.y[2] + n.x[2];
+        const R q = a.Qin[i * a.plane + o0];
+        const R *f = a.S + i * a.plane;
+        g[i] = i == 0 ? q : n.advance(f, i, f[o0], q);
+    }
+    R Fx, Fy;
+    if (WALLS && side >= 0) {  // Eq. 3.10 for the new f~ (force shift dt/2)
+        R u, v, wv[9];
+        wall_velocity(a, side, u, v);
+        load_force<R, FORCE>(a, jx, jy, Fx, Fy);
+        nee<R, FORCE>(a.c, g, Fx, Fy, a.c.half_dt, u, v, wv);
+#pragma unroll
+        for (int i = 0; i < 9; ++i) g[i] = wv[i];
+    }
+    const size_t o = (size_t)y * a.pitch + x;
+    if (LAST) {
+#pragma unroll
+        for (int i = 0; i < 9; ++i) a.Qout[i * a.plane + o] = g[i];
+        return;
+    }
+    load_force<R, FORCE>(a, x, y, Fx, Fy);
+    R P[9], Q[9];
+    prepare<R, FORCE>(a, g, Fx, Fy, P, Q);
+    chain_next();
+#pragma unroll
+    for (int i = 0; i < 9; ++i) {
+        a.P[i * a.plane + o] = P[i];
+        a.Qout[i * a.plane + o] = Q[i];
+    }
+}
+
+// One launch over all nodes; split_walls: the wall nodes in blocks of their
+// own.  chained: scheduled while the previous launch of the chain still runs.
+template <class R, class K>
+cudaError_t launch(K kernel, SplitArgs<R> a, bool split_walls, bool chained, cudaStream_t s)
+{
+    constexpr int nt = kThreads<R>;
+    const int wx = split_walls && a.wx, wy = split_walls && a.wy;
+    a.x0 = wx;
+    a.y0 = wy;
+    a.w = a.nx - 2 * wx;
+    a.h = a.ny - 2 * wy;
+    const int strips = (a.w + 63) / 64;
+    a.strip = (a.w + strips - 1) / strips;
+    a.strip_blocks = (int)(((long long)a.strip * a.h + nt - 1) / nt);
+    const long long walls = (wy ? 2ll * a.nx : 0) + (wx ? 2ll * a.h : 0);
+    a.wall_blocks = (int)((walls + nt - 1) / nt);
+    cudaLaunchConfig_t cfg{};
+    cfg.blockDim = dim3(nt);
+    cfg.gridDim = dim3((unsigned)(a.wall_blocks + a.strip_blocks * ((a.w + a.strip - 1) / a.strip)));
+    cfg.stream = s;
+    cudaLaunchAttribute at{};
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = chained ? 1 : 0;
+    return cudaLaunchKernelEx(&cfg, kernel, a);
+}
+
+template <class R, bool FORCE, bool WALLS>
+cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStream_t s)
+{
+    const R *bx = tabs, *by = tabs + 8 * (size_t)a.nx;                     // stage B (scale -h m)
+    const R *cxs = by + 8 * (size_t)a.ny, *cys = cxs + 8 * (size_t)a.nx;   // stage C (scale -dt m)
+    R *q[2] = {Q0, Q1};
+    a.Qout = q[0];
+    cudaError_t e = launch<R>(k_split_prepare<R, FORCE>, a, false, false, s);
+    for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
+        const bool last = k + 1 == nsteps;
+        a.tx = bx;
+        a.ty = by;
+        e = launch<R>(k_split_star<R, FORCE, WALLS>, a, WALLS, true, s);
+        if (e != cudaSuccess) break;
+        a.tx = cxs;
+        a.ty = cys;
+        a.Qin = q[k & 1];
+        a.Qout = last ? a.P : q[(k + 1) & 1];
+        e = last ? launch<R>(k_split_update<R, FORCE, WALLS, true>, a, WALLS, true, s)
+                 : launch<R>(k_split_update<R, FORCE, WALLS, false>, a, WALLS, true, s);
+    }
+    return e;
+}
+
+// Weights of the mixed difference at one node of an axis, times `scale`, for
+// velocity sign +1 or -1: {k + s, k, k - s, k - 2s}; `central`: next to a wall.
+// In FP32 the taps go on the grid of weight_grid (lattice.cuh), on which the
+// centre, minus their sum, is exact: the update of a constant is exactly zero.
+template <class R>
+void taps(const Stencil<R> &st, bool central, double scale, R out[4])
+{
+    double t[3] = {double(st.wm1) * scale, double(st.w1) * scale, double(st.w2) * scale};
+    if (central) {
+        t[0] = 0.5 * scale;
+        t[1] = -0.5 * scale;
+        t[2] = 0.0;
+    }
+    if (sizeof(R) == 4 && scale != 0.0) {
+        const double q = std::ldexp(1.0, std::ilogb(scale) - 21);
+        for (double &v : t) v = std::nearbyint(v / q) * q;
+    }
+    const R m1 = R(t[0]), p1 = R(t[1]), p2 = R(t[2]);
+    out[0] = m1;
+    out[1] = -((m1 + p1) + p2);
+    out[2] = p1;
+    out[3] = p2;
+}
+
+}  // namespace
+
+size_t split_table_bytes(int nx, int ny, size_t real_size) { return 16 * (size_t)(nx + ny) * real_size; }
+
+// The tables in the order bx, by, cx, cy: [n][2][4] each.
+template <class R>
+std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
+                                 double beta, double h, double dt)
+{
+    const Stencil<R> st = make_stencil<R>(beta);
+    std::vector<R> out;
+    out.reserve(16 * (mx.size() + my.size()));
+    auto axis = [&](const std::vector<double> &m, bool wall, double s) {
+        const int n = (int)m.size();
+        for (int k = 0; k < n; ++k)
+            for (int sign = 1; sign >= -1; sign -= 2) {
+                // the second-order upwind tap k - 2 s would leave the domain
+                const bool central = wall && (sign > 0 ? k < 2 : k > n - 3);
+                R t[4];
+                taps<R>(st, central, -s * double(R(m[k])), t);
+                out.insert(out.end(), t, t + 4);
+            }
+    };
+    axis(mx, wx, h);
+    axis(my, wy, h);
+    axis(mx, wx, dt);
+    axis(my, wy, dt);
+    return out;
+}
+template std::vector<float> make_split_tables<float>(const std::vector<double> &, const std::vector<double> &, bool,
+                                                     bool, double, double, double);
+template std::vector<double> make_split_tables<double>(const std::vector<double> &, const std::vector<double> &, bool,
+                                                       bool, double, double, double);
+
+// nsteps steps of the state in s.gin, in place.
+template <class R>
+cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream)
+{
+    if (nsteps <= 0) return cudaSuccess;
+    SplitArgs<R> a{};
+    a.P = const_cast<R *>(s.gin);
+    a.S = s.gout;
+    a.force = s.force;
+    a.nx = s.nx;
+    a.ny = s.ny;
+    a.pitch = s.pitch;
+    a.plane = s.plane;
+    a.wx = s.bc_x == FDLBM_WALL;
+    a.wy = s.bc_y == FDLBM_WALL;
+    for (int k = 0; k < 4; ++k)
+        for (int j = 0; j < 2; ++j) a.wall_u[k][j] = s.wall_u[k][j];
+    a.c = s.c;
+    a.keep_star = (R(1) - s.c.b_star) * R(0.5);
+    a.w_star[0] = s.c.b_star * wq<R>(0);
+    a.w_star[1] = s.c.b_star * wq<R>(1);
+    a.w_star[2] = s.c.b_star * wq<R>(5);
+    a.l_star[0] = s.c.b_star * LinearCoef<R>::c1;
+    a.l_star[1] = s.c.b_star * LinearCoef<R>::c2;
+    if (a.wx || a.wy)
+        return s.force ? run<R, true, true>(a, Q0, Q1, tables, nsteps, stream)
+                       : run<R, false, true>(a, Q0, Q1, tables, nsteps, stream);
+    return s.force ? run<R, true, false>(a, Q0, Q0, tables, nsteps, stream)
+                   : run<R, false, false>(a, Q0, Q0, tables, nsteps, stream);
+}
+template cudaError_t launch_split<float>(const StepArgs<float> &, float *, float *, const float *, int, cudaStream_t);
+template cudaError_t launch_split<double>(const StepArgs<double> &, double *, double *, const double *, int,
+                                          cudaStream_t);
+
+}  // namespace fdlbm
