@@ -76,11 +76,17 @@ enum { FDLBM_EQ_STANDARD = 0, FDLBM_EQ_INCOMPRESSIBLE = 1 };
  *          (there the walled and the periodic scheme compute the same values),
  *          and a second launch of the walls sweep covers the 4-node frame:
  *          two launches per step (fdlbm_kernels_per_step).
- * AUTO picks WARP where it applies (the fastest measured on GB300 for the
- * periodic 4096^2 throughput case), except on walled grids of fewer than
- * 1.5 M nodes, where the frame launch's fixed cost makes the walls sweep
- * faster, and SCALAR otherwise.  Asking for a variant that does not apply
- * returns FDLBM_EUNSUPPORTED; the values 2 to 4 are not used. */
+ * AUTO (with path AUTO and rows_per_cta 0) runs FP32 grids of small and medium
+ * size on the tile kernel (one launch per step, a tile of 32 x 16 nodes per
+ * block through all stages in shared memory), where it is the fastest measured
+ * on GB300: periodic grids under 0.8 M nodes (1.2 M with a force field, and
+ * where WARP does not apply), walled ones under 2.4 M (4 M with a force field,
+ * any size where WARP does not apply).  Beyond that it picks WARP where it
+ * applies and SCALAR otherwise; with path FUSED or a tile height given, WARP
+ * where it applies, except on walled grids of fewer than 1.5 M nodes, where the
+ * frame launch's fixed cost makes the walls sweep faster, and SCALAR otherwise.
+ * Asking for a variant that does not apply returns FDLBM_EUNSUPPORTED; the
+ * values 2 to 4 are not used. */
 enum { FDLBM_VARIANT_AUTO = 0, FDLBM_VARIANT_SCALAR = 1, FDLBM_VARIANT_WARP = 5 };
 enum { FDLBM_WALL_W = 0, FDLBM_WALL_E = 1, FDLBM_WALL_S = 2, FDLBM_WALL_N = 3 };
 /* Time-marching scheme (Sec. 2A):
@@ -328,9 +334,10 @@ long long fdlbm_batch_cells(fdlbm_batch_t b);        /* nodes of all cases */
 /* Advance every case by n steps (asynchronous on the batch stream). */
 fdlbm_status fdlbm_batch_step(fdlbm_batch_t b, int n);
 /* How fdlbm_batch_step advances the cases:
- *  FUSED       the fused sweeps with Eq. 3.10 inside them over tiles of every
- *              case: one launch per step for the T2S2-FDLBM1 cases and one for
- *              the T2S2-FDLBM2 cases (FP32 batches; the default there);
+ *  FUSED       the fused kernels with Eq. 3.10 inside them over tiles of every
+ *              case: one launch per step for the T2S2-FDLBM1 cases (the tile
+ *              kernel) and one for the T2S2-FDLBM2 cases (FP32 batches; the
+ *              default there);
  *  STAGED      one launch per stage and step of the staged kernels (the default
  *              otherwise);
  *  PERSISTENT  one cooperative launch for all the steps of a call (or of a graph

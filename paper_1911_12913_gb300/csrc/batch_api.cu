@@ -51,7 +51,7 @@ struct fdlbm_batch_ctx {
     // FUSED mode: the interiors of T2S2-FDLBM1 cases on the warp-tile kernel,
     // in groups of one kernel instance each (tiles [off, off + count) of the
     // tables), the frames of the walled ones (walls sweep in blocks of one
-    // warp, a group without and one with a force field), then the walls sweep
+    // warp, a group without and one with a force field), then the tile kernel
     // for the other T2S2-FDLBM1 cases (tiles [walls_off, blocks_s1)), then the
     // T2S2-FDLBM2 cases
     void *d_wargs = nullptr;  // 2 x ncases warp-tile argument blocks (tensor maps, scalars)
@@ -87,9 +87,10 @@ fdlbm_status bfail(fdlbm_batch_ctx *b, fdlbm_status s, const std::string &what)
 }
 
 // Host-side tables, uploaded to the device: for the staged kernels, node tiles
-// of block shape `blk`; for the fused sweep (fused_rows > 0), tiles of one
-// strip of the sweep's width by min(fused_rows, ny) rows (each case's tile
-// height goes into its argument block).
+// of block shape `blk`; for the fused kernels (fused_rows > 0), the tiles of the
+// tile kernel (FUSED mode, T2S2-FDLBM1), and for the sweeps tiles of one strip
+// of the sweep's width by min(fused_rows, ny) rows (each case's tile height goes
+// into its argument block).
 fdlbm_status build_tables(fdlbm_batch_ctx *b, dim3 blk, int fused_rows = 0)
 {
     const int n = (int)b->cases.size();
@@ -97,8 +98,8 @@ fdlbm_status build_tables(fdlbm_batch_ctx *b, dim3 blk, int fused_rows = 0)
     int total_wall = 0, total_blocks = 0, blocks_s1 = 0;
     bool any2 = false;
     // the tiles of T2S2-FDLBM1 cases first (in FUSED mode those on the
-    // warp-tile kernel, grouped by kernel instance, then those on the walls
-    // sweep), then those of T2S2-FDLBM2 cases; the fused batch runs each group
+    // warp-tile kernel, grouped by kernel instance, then those on the tile
+    // kernel), then those of T2S2-FDLBM2 cases; the fused batch runs each group
     // with its own launch
     const bool warp = fused_rows > 0 && b->mode == FDLBM_BATCH_FUSED;
     auto on_warp = [&](const fdlbm_ctx *h) {
@@ -153,6 +154,9 @@ fdlbm_status build_tables(fdlbm_batch_ctx *b, dim3 blk, int fused_rows = 0)
             if (b->wgroups.empty() || !(b->wgroups.back().kind == kinds[c]))
                 b->wgroups.push_back({kinds[c], total_blocks, 0});
             b->wgroups.back().count += tx * ty;
+        } else if (warp && h->scheme == FDLBM_SCHEME_T2S2_1) {
+            h->rows = 1;
+            tile_counts(h->nx, h->ny, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, &tx, &ty);
         } else if (fused_rows > 0) {
             h->rows = std::min(fused_rows, h->ny);
             tx = (h->nx + fused_tile_width_walls() - 1) / fused_tile_width_walls();
@@ -275,9 +279,10 @@ bool uses_fused_sweep(const fdlbm_batch_ctx *b)
            (b->mode == FDLBM_BATCH_PERSISTENT && fused_eligible(b) && all_scheme1(b));
 }
 
-// Tile height of the fused batch: minimise (waves) x (rows + 8) over the tiles
-// of all cases, as for a single grid, with the waves of the warp-tile launches
-// and of the walls sweep counted separately (they run one after the other).
+// Tile height of the fused batch's sweeps: minimise (waves) x (rows + 8) over the
+// tiles of all cases, as for a single grid, with the waves of the warp-tile
+// launches and of the scalar sweeps counted separately (they run one after the
+// other).  In FUSED mode the tile kernel's cases have no say.
 int fused_rows_model(const fdlbm_batch_ctx *b)
 {
     int dev = 0, sms = 152;
@@ -286,16 +291,17 @@ int fused_rows_model(const fdlbm_batch_ctx *b)
     const long long slots = (long long)std::max(1, fused_walls_blocks_per_sm<float>()) * sms;
     const long long wslots = (long long)std::max(1, fused_warp_blocks_per_sm()) * sms;
     const int W = fused_tile_width_walls(), WW = fused_warp_tile_width();
-    const bool warp = b->mode == FDLBM_BATCH_FUSED;
+    const bool fused = b->mode == FDLBM_BATCH_FUSED;
     int best = 64;
     double best_cost = 1e300;
     for (int rows = 1; rows <= 512; ++rows) {
         long long ctas = 0, wtiles = 0;
         for (const fdlbm_ctx *h : b->cases) {
             const int r = std::min(rows, h->ny), ty = (h->ny + r - 1) / r;
-            if (warp && h->scheme == FDLBM_SCHEME_T2S2_1 && h->variant == FDLBM_VARIANT_WARP)
+            const bool s1 = h->scheme == FDLBM_SCHEME_T2S2_1;
+            if (fused && s1 && h->variant == FDLBM_VARIANT_WARP)
                 wtiles += (long long)((h->nx + WW - 1) / WW) * ty;
-            else
+            else if (!fused || !s1)
                 ctas += (long long)((h->nx + W - 1) / W) * ty;
         }
         const double cost = (double)((ctas + slots - 1) / slots + (wtiles + wslots - 1) / wslots) * (rows + 8);
@@ -330,9 +336,7 @@ cudaError_t launch_steps(fdlbm_batch_ctx *b, int parity, int n)
                 e = launch_batched_warp(static_cast<const char *>(b->d_wargs) + p * wsz, b->tab.blk_case,
                                         b->tab.blk_start, g.off, g.count, g.kind, b->stream);
             }
-            if (e == cudaSuccess && nw > 0)
-                e = f32 ? launch_batched_fused<float>(b->tab, p, b->walls_off, nw, b->stream)
-                        : launch_batched_fused<double>(b->tab, p, b->walls_off, nw, b->stream);
+            if (e == cudaSuccess && nw > 0) e = launch_batched_tile(b->tab, p, b->walls_off, nw, b->stream);
             if (e == cudaSuccess && n2 > 0)
                 e = f32 ? launch_batched_fused_s2<float>(b->tab, p, n1, n2, b->stream)
                         : launch_batched_fused_s2<double>(b->tab, p, n1, n2, b->stream);
@@ -451,8 +455,13 @@ fdlbm_status autotune(fdlbm_batch_ctx *b)
     std::vector<TuneChoice> cand;
     if (uses_fused_sweep(b)) {
         const int r0 = fused_rows_model(b);
+        const bool sweeps = b->mode != FDLBM_BATCH_FUSED ||
+                            std::any_of(b->cases.begin(), b->cases.end(), [](const fdlbm_ctx *h) {
+                                return h->scheme != FDLBM_SCHEME_T2S2_1 || h->variant == FDLBM_VARIANT_WARP;
+                            });
         for (int r : {r0, std::max(1, r0 / 2), std::max(1, 3 * r0 / 4), std::min(512, 2 * r0)})
-            if (std::none_of(cand.begin(), cand.end(), [&](const TuneChoice &c) { return c.rows == r; }))
+            if ((sweeps || cand.empty()) &&
+                std::none_of(cand.begin(), cand.end(), [&](const TuneChoice &c) { return c.rows == r; }))
                 cand.push_back({dim3(128, 1), r});
     } else {
         for (const dim3 &d : {dim3(32, 8), dim3(64, 4), dim3(128, 2), dim3(32, 4), dim3(16, 16), dim3(256, 1)})

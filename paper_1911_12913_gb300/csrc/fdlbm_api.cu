@@ -104,6 +104,38 @@ bool use_split(const fdlbm_opts *o, int path)
            o->rows_per_cta == 0;
 }
 
+// Walled FP32 grids of fewer nodes run on the tile kernel rather than on the
+// warp tile and its frame (see use_tile).
+double tile_walled_nodes(const fdlbm_opts *o) { return o->has_force ? 4.0e6 : 2.4e6; }
+
+// T2S2-FDLBM1 in FP32 on the tile kernel (step_tile.cu) unless a tile height or
+// a kernel is asked for: a step of it lasts 4-5 us on the smallest grids, where
+// the sweeps walk a chain of ten dependent rows, and runs at 36-38 GLUPS (31
+// with a force field) on large ones.  us per step on GB300, tile kernel against
+// the one it replaces:
+//   walls sweep    257^2 4.9 / 9.8, 1025^2 29.2 / 51.2, 1000 x 513 forced channel 18.0 / 32.3
+//   scalar sweep   64^2 3.5 / 5.1, 768^2 16.4 / 20.5, 1024^2 27.0 / 29.1, 2048^2 110 / 97
+//   warp tile      64^2 3.5 / 9.3, 512^2 8.9 / 14.6, 768^2 16.4 / 18.5, 1024^2 27.0 / 26.1;
+//                  with a force field 256^2 4.2 / 13.5, 512^2 10.4 / 21.0, 1024^2 32.9 / 34.9
+//   warp tile and frame (about 28 us + 16 us per M nodes; forced 26 us per M)
+//                  1025^2 29.2 / 47.0, 2049^2 114 / 96, forced 2048 x 2049 134 / 136
+// The lines below lie where the two cross.  On periodic grids the warp tile, where
+// it applies, also keeps the thin ones that fill less than 0.7 of their tiles
+// (300 x 33: the choice that fdlbm_describe has always shown for it).
+bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
+{
+    if (o->scheme != FDLBM_SCHEME_T2S2_1 || o->precision != FDLBM_FP32_DEV || path != FDLBM_PATH_FUSED ||
+        o->path != FDLBM_PATH_AUTO || o->variant != FDLBM_VARIANT_AUTO || o->rows_per_cta != 0)
+        return false;
+    const double nodes = (double)g->nx * g->ny;
+    const bool warp = fused_warp_ok(g->nx, g->ny, g->bc_x == FDLBM_WALL);
+    if (walled(g)) return !warp || nodes < tile_walled_nodes(o);
+    if (!warp) return nodes < 1.2e6;
+    int tx, ty;
+    tile_counts(g->nx, g->ny, false, false, &tx, &ty);
+    return nodes < (o->has_force ? 1.2e6 : 0.8e6) && nodes >= 0.7 * 512.0 * tx * ty;
+}
+
 // Scratch fields a handle needs (see make_layout).
 int scratch_fields(const fdlbm_grid *g, const fdlbm_opts *o, int path, bool force_staged)
 {
@@ -205,6 +237,7 @@ cudaError_t launch_step(fdlbm_ctx *h, cudaStream_t s)
     if (h->precision == FDLBM_FP32_DEV) {
         auto a = step_args<float>(h);
         if (h->path == FDLBM_PATH_STAGED) return launch_staged(a, s);
+        if (h->tile) return launch_tile(a, s);
         if (h->variant == FDLBM_VARIANT_WARP) return launch_fused_warp(a, h->wmaps, h->cur, s);
         if (h->scheme == FDLBM_SCHEME_T2S2_2) return launch_fused_s2(a, s);
         if (walls) return launch_fused_walls(a, s);
@@ -498,8 +531,10 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     // a walled grid on the warp-tile kernel pays a fixed 25-35 us for its frame
     // launch (rows of the walls sweep are a chain of dependent work): below
     // about 1.5 M nodes the walls sweep alone is faster (measured on GB300:
-    // 1025^2 channel 40 us against 43, 2049^2 cavity 164 us against 107)
-    const bool small_walled = walled(g) && (long long)g->nx * g->ny < (3ll << 19);
+    // 1025^2 channel 40 us against 43, 2049^2 cavity 164 us against 107); in a
+    // batch the tile kernel takes the walls sweep's place
+    const double small_nodes = force_staged ? tile_walled_nodes(&o) : 1.5 * 1048576;
+    const bool small_walled = walled(g) && (double)g->nx * g->ny < small_nodes;
     if (variant == FDLBM_VARIANT_AUTO)
         variant = warp_ok && !small_walled ? FDLBM_VARIANT_WARP : FDLBM_VARIANT_SCALAR;
     mx.assign(g->nx, 0.0);
@@ -544,6 +579,7 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->adjoint = o.adjoint != 0;
     h->graph_steps = o.graph_steps > 0 ? o.graph_steps + (o.graph_steps & 1) : 0;
     h->split = !force_staged && use_split(&o, path);
+    h->tile = !force_staged && use_tile(g, &o, path);
     h->lay = make_layout(h->nx, h->ny, h->pitch, h->precision, h->has_force,
                          scratch_fields(g, &o, path, force_staged), h->split);
     cudaGetDevice(&h->device);
@@ -671,7 +707,7 @@ fdlbm_status fdlbm_create(const fdlbm_grid *g, const fdlbm_metrics *metrics, dou
         h->ws_bytes = h->lay.total;
     }
     st = handle_upload(h, mx, my);
-    if (st == FDLBM_OK && h->variant == FDLBM_VARIANT_WARP) {
+    if (st == FDLBM_OK && h->variant == FDLBM_VARIANT_WARP && !h->tile) {
         // tensor maps of both ping-pong buffers (and of the force field) for the
         // warp-tile kernel
         if (fused_warp_encode(&h->wmaps, reinterpret_cast<const float *>(h->ws + h->lay.state[0]),
@@ -875,6 +911,7 @@ int fdlbm_kernels_per_step(fdlbm_t h)
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
     if (h->split) return 2;  // and one more per fdlbm_step call (or graph replay)
     if (h->path == FDLBM_PATH_FUSED) {
+        if (h->tile) return 1;
         // a walled grid on the warp-tile kernel: the frame's launch and the interior's
         if (h->precision == FDLBM_FP32_DEV && h->variant == FDLBM_VARIANT_WARP && walls) {
             int interior = 0, frame = 0;
@@ -994,14 +1031,15 @@ const char *fdlbm_describe(fdlbm_t h)
         return h->desc.c_str();
     }
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
-    const char *kern = h->split                            ? "split"
+    const char *kern = h->tile                             ? "fused-tile"
+                       : h->split                          ? "split"
                        : h->path == FDLBM_PATH_STAGED      ? "staged"
                        : h->variant == FDLBM_VARIANT_WARP   ? "fused-warp"
                        : walls                              ? "fused-walls"
                                                             : "fused";
     h->desc = std::string(kern) + " " + prec;
-    if (!h->split) h->desc += " rows=" + std::to_string(h->rows);
-    if (walls && h->path == FDLBM_PATH_FUSED && h->variant == FDLBM_VARIANT_WARP) h->desc += " walls";
+    if (!h->split && !h->tile) h->desc += " rows=" + std::to_string(h->rows);
+    if (walls && h->path == FDLBM_PATH_FUSED && h->variant == FDLBM_VARIANT_WARP && !h->tile) h->desc += " walls";
     if (h->graph_steps) h->desc += " graph_steps=" + std::to_string(h->graph_steps);
     if (h->incomp) h->desc += " incompressible";
     return h->desc.c_str();

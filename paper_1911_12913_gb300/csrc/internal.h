@@ -78,6 +78,7 @@ struct fdlbm_ctx {
     bool in_batch = false;               // owned by a batch: stepped by fdlbm_batch_step
     bool adjoint = false;                // scratch for the adjoint step reserved
     bool split = false;                  // two launches per step (step_split.cu), in place
+    bool tile = false;                   // FP32 tile kernel (step_tile.cu)
     int graph_steps = 0;                 // steps per replayed CUDA graph (even), 0 = none
     fdlbm::WarpMaps wmaps{};             // tensor maps of the warp-tile kernel
     cudaGraph_t graph = nullptr;
@@ -175,9 +176,6 @@ template <class R>
 cudaError_t launch_fused_walls(const StepArgs<R> &a, cudaStream_t s);
 template <class R>
 int fused_walls_blocks_per_sm();
-template <class R>
-cudaError_t launch_batched_fused(const BatchTables &t, int parity, int blk_off, int nblocks,
-                                 cudaStream_t s);
 int fused_tile_width_walls();
 // step_split.cu (two launches per step, one node per thread; the state in
 // s.gin is advanced in place, s.gout is scratch)
@@ -187,6 +185,10 @@ std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vecto
                                  double beta, double h, double dt);
 template <class R>
 cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream);
+// step_tile.cu (FP32 T2S2-FDLBM1, one launch per step, a tile per block)
+void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty);
+cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s);
+cudaError_t launch_batched_tile(const BatchTables &t, int parity, int blk_off, int nblocks, cudaStream_t s);
 // step_staged.cu
 template <class R>
 cudaError_t launch_staged(const StepArgs<R> &a, cudaStream_t s);

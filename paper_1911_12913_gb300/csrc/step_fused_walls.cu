@@ -1,6 +1,6 @@
 // Fused T2S2-FDLBM1 step with walls, one launch per step: the sweep of
-// walls_sweep.cuh in blocks of 128 columns (120 outputs), for single grids,
-// batches and the persistent batch.
+// walls_sweep.cuh in blocks of 128 columns (120 outputs), for single grids and
+// the persistent batch.
 #include <cstdint>
 
 #include <algorithm>
@@ -40,33 +40,6 @@ __global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2) k_step_fused_walls
     const int y0 = blockIdx.y * a.rows;
     if (y0 >= a.ny) return;  // uniform over the block
     sweep_tile<R, FORCE>(a, sm, blockIdx.x * (NT - 2 * kHalo), y0);
-}
-
-// Batched: block b is tile (b - blk_start[c]) of case c = blk_case[b], with
-// strips[c] strips per row of tiles; the case's arguments (its own tile height
-// in .rows) are copied into shared memory first.
-template <class R>
-__global__ void __launch_bounds__(NT, sizeof(R) == 4 ? 3 : 2)
-    kb_step_fused_walls(const StepArgs<R> *cases, const int *blk_case, const int *blk_start,
-                        const int *strips, int blk_off)
-{
-    extern __shared__ __align__(16) unsigned char smem_raw[];
-    Smem<R> &sm = *reinterpret_cast<Smem<R> *>(smem_raw);
-    __shared__ __align__(16) unsigned char abuf[sizeof(StepArgs<R>)];
-    static_assert(sizeof(StepArgs<R>) % 4 == 0, "argument block is copied as 32-bit words");
-    const int bid = blk_off + blockIdx.x;
-    const int c = blk_case[bid];
-    {
-        const int *src = reinterpret_cast<const int *>(cases + c);
-        int *dst = reinterpret_cast<int *>(abuf);
-        for (int k = threadIdx.x; k < (int)(sizeof(StepArgs<R>) / 4); k += blockDim.x) dst[k] = src[k];
-    }
-    __syncthreads();
-    const StepArgs<R> &a = *reinterpret_cast<const StepArgs<R> *>(abuf);
-    const int lb = bid - blk_start[c], ns = strips[c];
-    const int y0 = (lb / ns) * a.rows;
-    if (y0 >= a.ny) return;  // uniform over the block
-    sweep_tile<R, true>(a, sm, (lb % ns) * (NT - 2 * kHalo), y0);
 }
 
 // Persistent batched: all tiles of all cases for nsteps steps in one
@@ -157,22 +130,6 @@ int fused_walls_blocks_per_sm()
     return n;
 }
 
-// One step of T2S2-FDLBM1 cases of a batch on the walls sweep (tiles
-// [blk_off, blk_off + nblocks) of its tables): one launch.
-template <class R>
-cudaError_t launch_batched_fused(const BatchTables &t, int parity, int blk_off, int nblocks,
-                                 cudaStream_t s)
-{
-    if (nblocks <= 0) return cudaSuccess;
-    constexpr size_t smem = sizeof(Smem<R>);
-    cudaError_t e = cudaFuncSetAttribute(kb_step_fused_walls<R>,
-                                         cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
-    kb_step_fused_walls<R><<<nblocks, NT, smem, s>>>(
-        static_cast<const StepArgs<R> *>(t.args[parity]), t.blk_case, t.blk_start, t.tiles_x, blk_off);
-    return cudaGetLastError();
-}
-
 int fused_tile_width_walls() { return NT - 2 * kHalo; }
 
 template <class R>
@@ -222,8 +179,6 @@ template cudaError_t launch_persistent_fused<float>(const BatchTables &, void *,
 template cudaError_t launch_persistent_fused<double>(const BatchTables &, void *, int, int,
                                                      cudaStream_t, unsigned);
 
-template cudaError_t launch_batched_fused<float>(const BatchTables &, int, int, int, cudaStream_t);
-template cudaError_t launch_batched_fused<double>(const BatchTables &, int, int, int, cudaStream_t);
 template cudaError_t launch_fused_walls<float>(const StepArgs<float> &, cudaStream_t);
 template cudaError_t launch_fused_walls<double>(const StepArgs<double> &, cudaStream_t);
 template int fused_walls_blocks_per_sm<float>();
