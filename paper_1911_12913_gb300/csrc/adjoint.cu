@@ -17,8 +17,8 @@
 // (dQ/dF)^T lam_Q at every node.  The transposed difference gathers from the
 // mirrored offsets, with the metric of the node it gathers from:
 //   (T^T lam)(k) = sum_j w_j m(k + s j) lam(k + s j).
-// Three kernels per step: recompute P; stage B adjoint (needs P and lam' in a
-// +-2 neighbourhood); stage A adjoint (needs lam_gs in a +-2 neighbourhood).
+// The sweep below runs FP64 handles, and FP32 ones whose buffers are not 8-byte
+// aligned; the others take the tile kernel (adjoint_tile.cu).
 #include <algorithm>
 #include <type_traits>
 

@@ -558,6 +558,10 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->bc_y = g->bc_y;
     std::memcpy(h->wall_u, g->wall_u, sizeof(h->wall_u));
     h->precision = o.precision;
+    auto one_value = [](const std::vector<double> &m) {
+        return std::all_of(m.begin(), m.end(), [&](double v) { return float(v) == float(m[0]); });
+    };
+    h->uniform = one_value(mx) && one_value(my);
     h->scheme = o.scheme;
     h->incomp = o.equilibrium == FDLBM_EQ_INCOMPRESSIBLE ? 1 : 0;
     h->nu = nu;
@@ -964,8 +968,11 @@ fdlbm_status fdlbm_adjoint_step(fdlbm_t h, const void *state_n, const void *lam_
     if (h->precision == FDLBM_FP32_DEV) {
         StepArgs<float> a = step_args<float>(h);
         a.gin = static_cast<const float *>(state_n);
-        e = launch_adjoint<float>(a, static_cast<const float *>(lam_next), static_cast<float *>(lam_prev),
-                                  a.P, a.Q, fB, dforce, h->stream);
+        const float *ln = static_cast<const float *>(lam_next);
+        float *lp = static_cast<float *>(lam_prev);
+        e = adjoint_tile_ok(state_n, lam_next, lam_prev)
+                ? launch_adjoint_tile(a, h->uniform, ln, lp, dforce, h->stream)
+                : launch_adjoint<float>(a, ln, lp, a.P, a.Q, fB, dforce, h->stream);
     } else {
         StepArgs<double> a = step_args<double>(h);
         a.gin = static_cast<const double *>(state_n);

@@ -78,6 +78,7 @@ struct fdlbm_ctx {
     bool in_batch = false;               // owned by a batch: stepped by fdlbm_batch_step
     bool adjoint = false;                // scratch for the adjoint step reserved
     bool split = false;                  // two launches per step (step_split.cu), in place
+    bool uniform = false;                // one metric value on each axis
     bool tile = false;                   // FP32 tile kernel (step_tile.cu)
     int graph_steps = 0;                 // steps per replayed CUDA graph (even), 0 = none
     fdlbm::WarpMaps wmaps{};             // tensor maps of the warp-tile kernel
@@ -208,6 +209,10 @@ cudaError_t launch_persistent_fused(const BatchTables &t, void *bar, int parity0
 template <class R>
 int persistent_fused_blocks_per_sm();
 size_t persistent_barrier_bytes();
+// adjoint_tile.cu (FP32)
+bool adjoint_tile_ok(const void *state, const void *lam_next, const void *lam_prev);
+cudaError_t launch_adjoint_tile(const StepArgs<float> &a, bool uniform, const float *lam_next, float *lam_prev,
+                                double *dforce, cudaStream_t s);
 // adjoint.cu
 template <class R>
 cudaError_t launch_adjoint(const StepArgs<R> &a, const R *lam_next, R *lam_prev, R *P, R *lgs,

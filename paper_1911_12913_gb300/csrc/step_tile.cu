@@ -22,19 +22,13 @@
 
 #include "internal.h"
 #include "packed.cuh"
+#include "tile.cuh"
 #include "walls_nodes.cuh"
 
 namespace fdlbm {
 namespace {
 
 using namespace packed;
-
-constexpr int kTX = 32, kTY = 16, kTP = kTX / 2;  // tile; pairs per row
-constexpr int kNT = kTP * kTY;                    // threads, one per pair of the tile
-constexpr int kAP = kTP + 4, kAR = kTY + 8;       // region of stage A: pairs per row, rows
-constexpr int kBP = kTP + 2, kBR = kTY + 4;       // region of stage B
-constexpr int kARing = kAP * kAR - kNT, kBRing = kBP * kBR - kNT;  // pairs around the tile
-static_assert(kARing <= kNT && kBRing <= kNT, "one pass over the ring");
 
 template <bool FORCE>
 struct TileSmem {
@@ -44,38 +38,6 @@ struct TileSmem {
     f2 F[FORCE ? 2 : 1][FORCE ? kAP * kAR : 1];
     float mx[2 * kAP], my[kAR];  // metrics of stage A's region
 };
-
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
-
-// Index k of an axis of n nodes: wrapped on a periodic axis, the nearest node
-// on a walled one.
-__device__ __forceinline__ int axis_index(int k, int n, bool wall)
-{
-    if (wall) return min(max(k, 0), n - 1);
-    if (k < 0) k += n;
-    if (k >= n) k -= n;
-    return (unsigned)k < (unsigned)n ? k : wrap_index(k, n);
-}
-
-// Pair c, row r of site q of the ring around the tile, in the region of
-// (kTP + H) pairs x (kTY + 2 H) rows: rows below and above, then the sides.
-template <int H>
-__device__ __forceinline__ void ring_site(int q, int &c, int &r)
-{
-    constexpr int W = kTP + H;  // H/2 pairs on each side
-    if (q < 2 * H * W) {
-        r = q / W;
-        c = q - r * W;
-        if (r >= H) r += kTY;
-    } else {
-        q -= 2 * H * W;
-        r = q / H;
-        c = q - r * H;
-        r += H;
-        if (c >= H / 2) c += kTP;
-    }
-}
 
 // Weights of the mixed difference in one axis times -s m, for the columns of
 // the pair (or one row, twice).  The plain form holds the scale; the edge form
@@ -479,18 +441,6 @@ __global__ void __launch_bounds__(kNT, kMinBlocks)
     __syncthreads();
     if (s->force) tile_step<true, true>(*s, smem_raw, u % nt, u / nt);
     else tile_step<false, true>(*s, smem_raw, u % nt, u / nt);
-}
-
-void chained_launch(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, dim3 grid, size_t smem, cudaStream_t s)
-{
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
 }
 
 }  // namespace

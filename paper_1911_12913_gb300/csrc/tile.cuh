@@ -1,0 +1,65 @@
+// Geometry and index helpers of the kernels that take a tile of the grid per
+// block through shared memory: the FP32 step (step_tile.cu) and its adjoint
+// (adjoint_tile.cu).  Threads work on pairs of neighbouring columns.
+#pragma once
+
+#include "lattice.cuh"
+
+namespace fdlbm {
+namespace {
+
+constexpr int kTX = 32, kTY = 16, kTP = kTX / 2;  // tile; pairs per row
+constexpr int kNT = kTP * kTY;                    // threads, one per pair of the tile
+constexpr int kAP = kTP + 4, kAR = kTY + 8;       // region of stage A: pairs per row, rows
+constexpr int kBP = kTP + 2, kBR = kTY + 4;       // region of stage B
+constexpr int kARing = kAP * kAR - kNT, kBRing = kBP * kBR - kNT;  // pairs around the tile
+static_assert(kARing <= kNT && kBRing <= kNT, "one pass over the ring");
+
+__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
+__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+
+// Index k of an axis of n nodes: wrapped on a periodic axis, the nearest node
+// on a walled one.
+__device__ __forceinline__ int axis_index(int k, int n, bool wall)
+{
+    if (wall) return min(max(k, 0), n - 1);
+    if (k < 0) k += n;
+    if (k >= n) k -= n;
+    return (unsigned)k < (unsigned)n ? k : wrap_index(k, n);
+}
+
+// Pair c, row r of site q of the ring around the tile, in the region of
+// (kTP + H) pairs x (kTY + 2 H) rows: rows below and above, then the sides.
+template <int H>
+__device__ __forceinline__ void ring_site(int q, int &c, int &r)
+{
+    constexpr int W = kTP + H;  // H/2 pairs on each side
+    if (q < 2 * H * W) {
+        r = q / W;
+        c = q - r * W;
+        if (r >= H) r += kTY;
+    } else {
+        q -= 2 * H * W;
+        r = q / H;
+        c = q - r * H;
+        r += H;
+        if (c >= H / 2) c += kTP;
+    }
+}
+
+// A launch of kNT threads per block that may start while the previous one on the
+// stream still runs; its blocks call chain_wait before they touch its results.
+inline void chained_launch(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, dim3 grid, size_t smem, cudaStream_t s)
+{
+    cfg.gridDim = grid;
+    cfg.blockDim = dim3(kNT);
+    cfg.dynamicSmemBytes = smem;
+    cfg.stream = s;
+    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
+    at.val.programmaticStreamSerializationAllowed = 1;
+    cfg.attrs = &at;
+    cfg.numAttrs = 1;
+}
+
+}  // namespace
+}  // namespace fdlbm
