@@ -105,8 +105,13 @@ bool use_split(const fdlbm_opts *o, int path)
 }
 
 // Walled FP32 grids of fewer nodes run on the tile kernel rather than on the
-// warp tile and its frame (see use_tile).
-double tile_walled_nodes(const fdlbm_opts *o) { return o->has_force ? 4.0e6 : 2.4e6; }
+// warp tile and its frame (see use_tile; in a batch the frame is a walls sweep,
+// whose fixed cost is higher).
+double tile_walled_nodes(const fdlbm_opts *o, bool batch)
+{
+    if (batch) return o->has_force ? 4.0e6 : 2.4e6;
+    return o->has_force ? 1.7e6 : 1.35e6;
+}
 
 // T2S2-FDLBM1 in FP32 on the tile kernel (step_tile.cu) unless a tile height or
 // a kernel is asked for: a step of it lasts 4-5 us on the smallest grids, where
@@ -117,8 +122,11 @@ double tile_walled_nodes(const fdlbm_opts *o) { return o->has_force ? 4.0e6 : 2.
 //   scalar sweep   64^2 3.5 / 5.1, 768^2 16.4 / 20.5, 1024^2 27.0 / 29.1, 2048^2 110 / 97
 //   warp tile      64^2 3.5 / 9.3, 512^2 8.9 / 14.6, 768^2 16.4 / 18.5, 1024^2 27.0 / 26.1;
 //                  with a force field 256^2 4.2 / 13.5, 512^2 10.4 / 21.0, 1024^2 32.9 / 34.9
-//   warp tile and frame (about 28 us + 16 us per M nodes; forced 26 us per M)
-//                  1025^2 29.2 / 47.0, 2049^2 114 / 96, forced 2048 x 2049 134 / 136
+//   warp tile, frame on the tile kernel
+//                  1281^2 48.6 / 43.1, 2049^2 115 / 81; forced 1024 x 1025 34.5 / 44,
+//                  1536 x 1537 78.9 / 68.1
+//   warp tile, frame as a walls sweep (a batch)
+//                  1025^2 29.2 / 44.5, 2049^2 115 / 95, forced 2048 x 2049 134 / 137
 // The lines below lie where the two cross.  On periodic grids the warp tile, where
 // it applies, also keeps the thin ones that fill less than 0.7 of their tiles
 // (300 x 33: the choice that fdlbm_describe has always shown for it).
@@ -129,7 +137,7 @@ bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
         return false;
     const double nodes = (double)g->nx * g->ny;
     const bool warp = fused_warp_ok(g->nx, g->ny, g->bc_x == FDLBM_WALL);
-    if (walled(g)) return !warp || nodes < tile_walled_nodes(o);
+    if (walled(g)) return !warp || nodes < tile_walled_nodes(o, false);
     if (!warp) return nodes < 1.2e6;
     int tx, ty;
     tile_counts(g->nx, g->ny, false, false, &tx, &ty);
@@ -238,7 +246,7 @@ cudaError_t launch_step(fdlbm_ctx *h, cudaStream_t s)
         auto a = step_args<float>(h);
         if (h->path == FDLBM_PATH_STAGED) return launch_staged(a, s);
         if (h->tile) return launch_tile(a, s);
-        if (h->variant == FDLBM_VARIANT_WARP) return launch_fused_warp(a, h->wmaps, h->cur, s);
+        if (h->variant == FDLBM_VARIANT_WARP) return launch_fused_warp(a, h->wmaps, h->cur, h->tile_frame, s);
         if (h->scheme == FDLBM_SCHEME_T2S2_2) return launch_fused_s2(a, s);
         if (walls) return launch_fused_walls(a, s);
         return launch_fused(a, s);
@@ -528,12 +536,12 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
                          fused_warp_ok(g->nx, g->ny, g->bc_x == FDLBM_WALL);
     if (o.variant == FDLBM_VARIANT_WARP && !warp_ok) return FDLBM_EUNSUPPORTED;
     int variant = o.variant;
-    // a walled grid on the warp-tile kernel pays a fixed 25-35 us for its frame
-    // launch (rows of the walls sweep are a chain of dependent work): below
-    // about 1.5 M nodes the walls sweep alone is faster (measured on GB300:
-    // 1025^2 channel 40 us against 43, 2049^2 cavity 164 us against 107); in a
-    // batch the tile kernel takes the walls sweep's place
-    const double small_nodes = force_staged ? tile_walled_nodes(&o) : 1.5 * 1048576;
+    // a walled grid on the warp-tile kernel pays a fixed cost for its frame
+    // launch: smaller ones run on the tile kernel, or, where a path or a tile
+    // height is asked for, below about 1.5 M nodes on the walls sweep
+    // (2049^2 cavity 164 us per step against 95 on the warp tile)
+    const bool auto_all = o.path == FDLBM_PATH_AUTO && o.rows_per_cta == 0;
+    const double small_nodes = force_staged || auto_all ? tile_walled_nodes(&o, force_staged) : 1.5 * 1048576;
     const bool small_walled = walled(g) && (double)g->nx * g->ny < small_nodes;
     if (variant == FDLBM_VARIANT_AUTO)
         variant = warp_ok && !small_walled ? FDLBM_VARIANT_WARP : FDLBM_VARIANT_SCALAR;
@@ -584,6 +592,7 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->graph_steps = o.graph_steps > 0 ? o.graph_steps + (o.graph_steps & 1) : 0;
     h->split = !force_staged && use_split(&o, path);
     h->tile = !force_staged && use_tile(g, &o, path);
+    h->tile_frame = !force_staged && walled(g) && s1 && o.variant == FDLBM_VARIANT_AUTO;
     h->lay = make_layout(h->nx, h->ny, h->pitch, h->precision, h->has_force,
                          scratch_fields(g, &o, path, force_staged), h->split);
     cudaGetDevice(&h->device);

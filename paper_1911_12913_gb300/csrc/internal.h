@@ -79,6 +79,7 @@ struct fdlbm_ctx {
     bool adjoint = false;                // scratch for the adjoint step reserved
     bool split = false;                  // two launches per step (step_split.cu), in place
     bool uniform = false;                // one metric value on each axis
+    bool tile_frame = false;             // warp tile: the frame on the tile kernel
     bool tile = false;                   // FP32 tile kernel (step_tile.cu)
     int graph_steps = 0;                 // steps per replayed CUDA graph (even), 0 = none
     fdlbm::WarpMaps wmaps{};             // tensor maps of the warp-tile kernel
@@ -130,7 +131,8 @@ cudaError_t launch_batched_fused_s2(const BatchTables &t, int parity, int blk_of
 bool fused_warp_ok(int nx, int ny, bool wall_x);
 cudaError_t fused_warp_encode(WarpMaps *m, const float *state0, const float *state1,
                               const float *force, int nx, int ny, int pitch, size_t plane);
-cudaError_t launch_fused_warp(const StepArgs<float> &a, const WarpMaps &maps, int cur,
+// tile_frame: the frame of a walled T2S2-FDLBM1 grid on the tile kernel (else the walls sweep).
+cudaError_t launch_fused_warp(const StepArgs<float> &a, const WarpMaps &maps, int cur, bool tile_frame,
                               cudaStream_t s);
 // Frame geometry of a walled grid split between the warp-tile kernel (the
 // interior rectangle [xoff, xend) x [yoff, yend)) and a walls sweep in blocks
@@ -189,6 +191,7 @@ cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, in
 // step_tile.cu (FP32 T2S2-FDLBM1, one launch per step, a tile per block)
 void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty);
 cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s);
+cudaError_t launch_frame_tile(const StepArgs<float> &a, int x0, int x1, int y0, int y1, cudaStream_t s);
 cudaError_t launch_batched_tile(const BatchTables &t, int parity, int blk_off, int nblocks, cudaStream_t s);
 // step_staged.cu
 template <class R>

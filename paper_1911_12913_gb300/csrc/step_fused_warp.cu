@@ -920,7 +920,7 @@ WarpKind warp_kind(const StepArgs<float> &s)
     return k;
 }
 
-cudaError_t launch_fused_warp(const StepArgs<float> &s, const WarpMaps &maps, int cur,
+cudaError_t launch_fused_warp(const StepArgs<float> &s, const WarpMaps &maps, int cur, bool tile_frame,
                               cudaStream_t stream)
 {
     if (s.force && !maps.has_force) return cudaErrorInvalidValue;
@@ -931,6 +931,8 @@ cudaError_t launch_fused_warp(const StepArgs<float> &s, const WarpMaps &maps, in
         const FrameGeom g{a.s.nx, a.s.ny, a.s.wx, a.s.wy, a.s.xoff, a.s.xend, a.s.yoff, a.s.yend, a.s.erows,
                           a.s.nframe};
         e = launch_frame_s2(g, s, stream);
+    } else if (a.s.nframe > 0 && tile_frame) {
+        e = launch_frame_tile(s, a.s.xoff, a.s.xend, a.s.yoff, a.s.yend, stream);
     } else if (a.s.nframe > 0) {
         e = s.force ? launch_frame_t<true>(a.s, s, stream) : launch_frame_t<false>(a.s, s, stream);
     }

@@ -18,6 +18,13 @@
 // whose weight is zero next to a wall where it would leave the domain.  Outside
 // a walled domain, loads read the nearest node; zero weights meet those values,
 // which are finite.
+//
+// What bounds it: at 1024^2 (27 us per step, 39 GLUPS) the shared-memory pipe,
+// about 65 % busy with 38 64-bit loads per pair and stage; issue slots 43 % busy.
+// The tile's halo costs 1.9 times stage A and 1.4 times stage B.  On small grids
+// it is one tile's latency: 64^2 3.5 us per step, 257^2 cavity 4.9 (walls sweep
+// 9.8).  Tried: two rows per thread (tile 32 x 32, 128 registers) 2048^2 122 us
+// against 110; more threads for the ring (384, 512) 1024^2 30 and 42 against 27.
 #include <algorithm>
 
 #include "internal.h"
@@ -46,7 +53,13 @@ struct Diff {
     f2 k1, k2p, k2n;
 };
 
-template <bool FORCE>
+// An output rectangle [x0, x1) x [y0, y1) that another launch writes.
+struct Rect {
+    int x0, x1, y0, y1;
+};
+
+// MASK: the frame of a walled grid around the warp-tile kernel's interior.
+template <bool FORCE, bool MASK = false>
 struct Tile {
     using Smem = TileSmem<FORCE>;
     const StepArgs<float> &a;
@@ -54,6 +67,7 @@ struct Tile {
     const int x0, y0, t;
     const bool wx, wy;
     const bool inside;  // no column of stage A's region lies outside [0, nx)
+    Rect skip;          // MASK: nodes that are not stored
     f2 w[4];  // mixed weights at +1, 0, -1, -2
     f2 rho0;
 
@@ -361,8 +375,12 @@ struct Tile {
         stage_c<EDGE>(p, r, Q);
         const int x = x0 + 2 * p, y = y0 + r;
         const bool row = wy ? y >= 1 && y <= a.ny - 2 : y < a.ny;
-        const bool lo = wx ? x >= 1 && x <= a.nx - 2 : x < a.nx;
-        const bool hi = wx ? x + 1 <= a.nx - 2 : x + 1 < a.nx;
+        bool lo = wx ? x >= 1 && x <= a.nx - 2 : x < a.nx;
+        bool hi = wx ? x + 1 <= a.nx - 2 : x + 1 < a.nx;
+        if (MASK && y >= skip.y0 && y < skip.y1) {
+            lo = lo && (x < skip.x0 || x >= skip.x1);
+            hi = hi && (x + 1 < skip.x0 || x + 1 >= skip.x1);
+        }
         float *dst = a.gout + (size_t)y * a.pitch + x;
         if (row && lo && hi) {
 #pragma unroll
@@ -422,6 +440,44 @@ __global__ void __launch_bounds__(kNT, kMinBlocks) k_step_tile(const __grid_cons
     tile_step<FORCE, WALLS>(a, smem_raw, blockIdx.x, blockIdx.y);
 }
 
+// The frame of a walled grid: the tiles that hold nodes outside `skip`, the
+// interior rectangle of the warp-tile kernel.  One wave of blocks lasts about
+// 10 us, where the walls sweep in blocks of one warp walks a chain of twelve rows
+// and more in 25 us (2049^2 cavity 95 -> 81 us per step, 4097^2 279 -> 265, forced
+// 2048 x 2049 channel 137 -> 113).  On a walled x axis those are the
+// first column of tiles and the ones from `east` on, then on a walled y axis the
+// first row and the ones from `north` on.
+struct FrameTiles {
+    Rect skip;
+    int tx, ty, east, north;  // tiles of the grid; first frame column and row on the far sides
+    int cols, rows;           // frame columns (ty tiles each) and rows (of the other columns)
+};
+
+template <bool FORCE>
+__global__ void __launch_bounds__(kNT, kMinBlocks)
+    k_frame_tile(const __grid_constant__ StepArgs<float> a, const __grid_constant__ FrameTiles f)
+{
+    extern __shared__ __align__(16) unsigned char smem_raw[];
+    int b = blockIdx.x, bx, by;
+    if (b < f.cols * f.ty) {
+        bx = b / f.ty;
+        by = b - bx * f.ty;
+        if (bx > 0) bx += f.east - 1;
+    } else {
+        b -= f.cols * f.ty;
+        const int w = f.tx - f.cols;  // the columns that are not in the frame
+        by = b / w;
+        bx = b - by * w + (f.cols > 0 ? 1 : 0);
+        if (by > 0) by += f.north - 1;
+    }
+    Tile<FORCE, true> tile(a, *reinterpret_cast<TileSmem<FORCE> *>(smem_raw), bx, by);
+    tile.skip = f.skip;
+    tile.metrics();
+    chain_wait();
+    tile.template go<true>();
+    chain_next();
+}
+
 // Batched: block b is tile (b - blk_start[c]) of case c = blk_case[b], tiles_x[c]
 // tiles per row; the case's arguments are copied into shared memory first.
 constexpr size_t kArgsOff = (sizeof(TileSmem<true>) + 15) / 16 * 16;
@@ -466,6 +522,28 @@ cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s)
     cudaLaunchAttribute at{};
     chained_launch(cfg, at, dim3(tx, ty), smem, s);
     return cudaLaunchKernelEx(&cfg, kern, a);
+}
+
+// The nodes of a walled grid outside the rectangle [x0, x1) x [y0, y1).
+cudaError_t launch_frame_tile(const StepArgs<float> &a, int x0, int x1, int y0, int y1, cudaStream_t s)
+{
+    const bool wx = a.bc_x == FDLBM_WALL, wy = a.bc_y == FDLBM_WALL;
+    FrameTiles f{{x0, x1, y0, y1}};
+    tile_counts(a.nx, a.ny, wx, wy, &f.tx, &f.ty);
+    // (a rectangle that is empty, or ends in the first tile: every tile is frame)
+    const bool none = x1 <= x0 || y1 <= y0;
+    f.east = none ? 1 : std::min(f.tx, std::max(1, x1 / kTX));
+    f.north = none ? 1 : std::min(f.ty, std::max(1, y1 / kTY));
+    f.cols = wx || none ? 1 + f.tx - f.east : 0;
+    f.rows = wy && f.cols < f.tx ? 1 + f.ty - f.north : 0;
+    const size_t smem = a.force ? sizeof(TileSmem<true>) : sizeof(TileSmem<false>);
+    auto kern = a.force ? k_frame_tile<true> : k_frame_tile<false>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    cudaLaunchConfig_t cfg{};
+    cudaLaunchAttribute at{};
+    chained_launch(cfg, at, dim3(f.cols * f.ty + f.rows * (f.tx - f.cols)), smem, s);
+    return cudaLaunchKernelEx(&cfg, kern, a, f);
 }
 
 // Tiles [blk_off, blk_off + nblocks) of the batch's tables.
