@@ -27,6 +27,13 @@ import torch
 from .solver import FDLBM
 
 
+def _buffer(solver: FDLBM):
+    """A state buffer whose contents do not matter (every value that is read is
+    written first)."""
+    pitch, dtype = solver.layout()
+    return torch.empty((9, solver.ny, pitch), dtype=dtype, device=solver.device)
+
+
 def _forward(solver: FDLBM, force, nsteps: int):
     """Run nsteps from the solver's current state under the force already set,
     keeping the checkpoints."""
@@ -34,11 +41,11 @@ def _forward(solver: FDLBM, force, nsteps: int):
     ckpts = []
     done = 0
     while done < nsteps:
-        ckpts.append(solver.save_state(solver.new_buffer()))
+        ckpts.append(solver.save_state(_buffer(solver)))
         n = min(k, nsteps - done)
         solver.step(n)
         done += n
-    final = solver.save_state(solver.new_buffer())
+    final = solver.save_state(_buffer(solver))
     _, ux, uy = solver.moments(device=True)
     return ckpts, final, k, torch.stack([ux, uy])
 
@@ -46,18 +53,18 @@ def _forward(solver: FDLBM, force, nsteps: int):
 def _reverse(s: FDLBM, ckpts, final, nsteps: int, k: int, grad_u, shape):
     """The adjoint sweep: (d/d force, cotangent of the initial state)."""
     dforce = torch.zeros(shape, dtype=torch.float64, device=s.device)
-    lam = s.new_buffer()
-    lam2 = s.new_buffer()
+    lam = _buffer(s)
+    lam2 = _buffer(s)
     keep = s.moments_vjp(final, grad_u, lam, dforce)
-    seg = [s.new_buffer() for _ in range(k)]
+    seg = [None] + [_buffer(s) for _ in range(min(k, nsteps) - 1)]
     for c in range(len(ckpts) - 1, -1, -1):
         start = c * k
         n = min(k, nsteps - start)
-        s.load_state(ckpts[c])
-        for j in range(n):
+        seg[0] = ckpts[c]  # the segment's first state
+        s.load_state(seg[0])
+        for j in range(1, n):
+            s.step(1)
             s.save_state(seg[j])
-            if j + 1 < n:
-                s.step(1)
         for j in range(n - 1, -1, -1):
             s.adjoint_step(seg[j], lam, lam2, dforce)
             lam, lam2 = lam2, lam
