@@ -521,10 +521,7 @@ cudaError_t launch_adjoint_tile(const StepArgs<float> &a, bool uniform, const fl
                         : (uniform ? k_adj_tile<false, true> : k_adj_tile<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjSmem));
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    chained_launch(cfg, at, dim3((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY), sizeof(AdjSmem), s);
-    return cudaLaunchKernelEx(&cfg, kern, q);
+    return chained_launch(kern, dim3((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY), kNT, sizeof(AdjSmem), s, q);
 }
 
 }  // namespace fdlbm

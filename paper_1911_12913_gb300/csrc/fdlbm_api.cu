@@ -110,7 +110,7 @@ bool use_split(const fdlbm_opts *o, int path)
 double tile_walled_nodes(const fdlbm_opts *o, bool batch)
 {
     if (batch) return o->has_force ? 4.0e6 : 2.4e6;
-    return o->has_force ? 1.7e6 : 1.35e6;
+    return o->has_force ? 1.7e6 : 1.25e6;
 }
 
 // T2S2-FDLBM1 in FP32 on the tile kernel (step_tile.cu) unless a tile height or
@@ -120,11 +120,12 @@ double tile_walled_nodes(const fdlbm_opts *o, bool batch)
 // the one it replaces:
 //   walls sweep    257^2 4.9 / 9.8, 1025^2 29.2 / 51.2, 1000 x 513 forced channel 18.0 / 32.3
 //   scalar sweep   64^2 3.5 / 5.1, 768^2 16.4 / 20.5, 1024^2 27.0 / 29.1, 2048^2 110 / 97
-//   warp tile      64^2 3.5 / 9.3, 512^2 8.9 / 14.6, 768^2 16.4 / 18.5, 1024^2 27.0 / 26.1;
-//                  with a force field 256^2 4.2 / 13.5, 512^2 10.4 / 21.0, 1024^2 32.9 / 34.9
+//   warp tile      64^2 3.5 / 9.3, 512^2 9.0 / 12.8, 768^2 16.4 / 16.8, 896^2 19.5 / 19.5,
+//                  1024^2 27.0 / 23.2; with a force field 256^2 4.2 / 13.5, 768^2
+//                  19.1 / 24.3, 1024^2 32.8 / 32.1, 1088^2 39.0 / 39.9
 //   warp tile, frame on the tile kernel
-//                  1281^2 48.6 / 43.1, 2049^2 115 / 81; forced 1024 x 1025 34.5 / 44,
-//                  1536 x 1537 78.9 / 68.1
+//                  1155^2 39.9 / 36, 2049^2 115 / 79; forced 1280 x 1281 55.7 / 54,
+//                  1536 x 1537 78.9 / 68
 //   warp tile, frame as a walls sweep (a batch)
 //                  1025^2 29.2 / 44.5, 2049^2 115 / 95, forced 2048 x 2049 134 / 137
 // The lines below lie where the two cross.  On periodic grids the warp tile, where

@@ -58,6 +58,7 @@
 
 #include <cuda.h>
 
+#include "chain.cuh"
 #include "internal.h"
 #include "packed.cuh"
 #include "tma.cuh"
@@ -371,6 +372,7 @@ __device__ __forceinline__ void warp_tile(const ArgsS &a, const CUtensorMap *tin
         mbar_init_fence();
     }
     __syncwarp();
+    chain_wait();  // nothing before this reads the previous step's results
     for (int s = 0; s < kStages && s < iters; ++s) issue(s, s);
 
     f2 Pw[9][5];  // fbar^{+,h} of the lane's columns, slot = iteration mod 5
@@ -582,6 +584,7 @@ __device__ __forceinline__ void warp_tile(const ArgsS &a, const CUtensorMap *tin
         if (k + 3 < iters) row(std::integral_constant<int, 3>{}, k + 3);
         if (k + 4 < iters) row(std::integral_constant<int, 4>{}, k + 4);
     }
+    chain_next();
     if (timed_out) {
         // the last copy into slot s was issued at iteration s + 3 n < iters, in
         // phase n; wait (bounded) for it before the shared memory is released
@@ -763,6 +766,9 @@ cudaError_t fused_warp_encode(WarpMaps *m, const float *state0, const float *sta
     return cudaSuccess;
 }
 
+// Chained: a step's barriers, metrics and weights are set up while the previous
+// step's last blocks run (1024^2 26.1 -> 23.2 us per step, 2048^2 69.8 -> 67.4,
+// 4096^2 247 -> 245, T2S2-FDLBM2 2048^2 102 -> 98).
 template <bool INC, bool GRID, bool FORCE, bool S2>
 cudaError_t launch_t(const ArgsW &a, dim3 grid, cudaStream_t stream)
 {
@@ -770,8 +776,7 @@ cudaError_t launch_t(const ArgsW &a, dim3 grid, cudaStream_t stream)
     auto kern = k_step_fused_warp<INC, GRID, FORCE, S2>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    kern<<<grid, kLanes, smem, stream>>>(a);
-    return cudaGetLastError();
+    return chained_launch(kern, grid, kLanes, smem, stream, a);
 }
 
 template <bool FORCE>

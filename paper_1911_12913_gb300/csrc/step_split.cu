@@ -30,6 +30,7 @@
 #include <cmath>
 #include <vector>
 
+#include "chain.cuh"
 #include "internal.h"
 #include "walls_nodes.cuh"
 
@@ -43,13 +44,10 @@ namespace {
 template <class R>
 constexpr int kThreads = sizeof(R) == 8 ? 32 : 128;
 
-// Wait for the previous launch of the chain (its results are visible after
-// this); let the next one's blocks be scheduled.  The second comes after a
-// warp's arithmetic: at the start of the kernel, the waiting blocks of the next
-// launch took SM slots unevenly (257^2 periodic FP64: 31.4 us per step against
-// 51.6; without the chain attribute 35.2).
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
+// The launches of a call are chained (chain.cuh).  Letting the next one's blocks
+// in at the start of the kernel instead of after a warp's arithmetic made them
+// take SM slots unevenly (257^2 periodic FP64: 51.6 us per step against 31.4;
+// without the chain attribute 35.2).
 
 template <class R>
 struct SplitArgs {
@@ -446,16 +444,10 @@ cudaError_t launch(K kernel, SplitArgs<R> a, bool split_walls, bool chained, cud
     a.strip_blocks = (int)(((long long)a.strip * a.h + nt - 1) / nt);
     const long long walls = (wy ? 2ll * a.nx : 0) + (wx ? 2ll * a.h : 0);
     a.wall_blocks = (int)((walls + nt - 1) / nt);
-    cudaLaunchConfig_t cfg{};
-    cfg.blockDim = dim3(nt);
-    cfg.gridDim = dim3((unsigned)(a.wall_blocks + a.strip_blocks * ((a.w + a.strip - 1) / a.strip)));
-    cfg.stream = s;
-    cudaLaunchAttribute at{};
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = chained ? 1 : 0;
-    return cudaLaunchKernelEx(&cfg, kernel, a);
+    const dim3 grid((unsigned)(a.wall_blocks + a.strip_blocks * ((a.w + a.strip - 1) / a.strip)));
+    if (chained) return chained_launch(kernel, grid, nt, 0, s, a);
+    kernel<<<grid, nt, 0, s>>>(a);
+    return cudaGetLastError();
 }
 
 template <class R, bool FORCE, bool WALLS>

@@ -518,10 +518,7 @@ cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     int tx, ty;
     tile_counts(a.nx, a.ny, a.bc_x == FDLBM_WALL, a.bc_y == FDLBM_WALL, &tx, &ty);
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    chained_launch(cfg, at, dim3(tx, ty), smem, s);
-    return cudaLaunchKernelEx(&cfg, kern, a);
+    return chained_launch(kern, dim3(tx, ty), kNT, smem, s, a);
 }
 
 // The nodes of a walled grid outside the rectangle [x0, x1) x [y0, y1).
@@ -540,10 +537,7 @@ cudaError_t launch_frame_tile(const StepArgs<float> &a, int x0, int x1, int y0, 
     auto kern = a.force ? k_frame_tile<true> : k_frame_tile<false>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    chained_launch(cfg, at, dim3(f.cols * f.ty + f.rows * (f.tx - f.cols)), smem, s);
-    return cudaLaunchKernelEx(&cfg, kern, a, f);
+    return chained_launch(kern, dim3(f.cols * f.ty + f.rows * (f.tx - f.cols)), kNT, smem, s, a, f);
 }
 
 // Tiles [blk_off, blk_off + nblocks) of the batch's tables.
@@ -553,11 +547,9 @@ cudaError_t launch_batched_tile(const BatchTables &t, int parity, int blk_off, i
     constexpr size_t smem = kArgsOff + sizeof(StepArgs<float>);
     cudaError_t e = cudaFuncSetAttribute(kb_step_tile, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
     if (e != cudaSuccess) return e;
-    cudaLaunchConfig_t cfg{};
-    cudaLaunchAttribute at{};
-    chained_launch(cfg, at, dim3(nblocks), smem, s);
-    return cudaLaunchKernelEx(&cfg, kb_step_tile, static_cast<const StepArgs<float> *>(t.args[parity]), t.blk_case,
-                              t.blk_start, t.tiles_x, blk_off);
+    return chained_launch(kb_step_tile, dim3(nblocks), kNT, smem, s,
+                          static_cast<const StepArgs<float> *>(t.args[parity]), t.blk_case, t.blk_start, t.tiles_x,
+                          blk_off);
 }
 
 }  // namespace fdlbm

@@ -3,6 +3,7 @@
 // (adjoint_tile.cu).  Threads work on pairs of neighbouring columns.
 #pragma once
 
+#include "chain.cuh"
 #include "lattice.cuh"
 
 namespace fdlbm {
@@ -14,9 +15,6 @@ constexpr int kAP = kTP + 4, kAR = kTY + 8;       // region of stage A: pairs pe
 constexpr int kBP = kTP + 2, kBR = kTY + 4;       // region of stage B
 constexpr int kARing = kAP * kAR - kNT, kBRing = kBP * kBR - kNT;  // pairs around the tile
 static_assert(kARing <= kNT && kBRing <= kNT, "one pass over the ring");
-
-__device__ __forceinline__ void chain_wait() { asm volatile("griddepcontrol.wait;" ::: "memory"); }
-__device__ __forceinline__ void chain_next() { asm volatile("griddepcontrol.launch_dependents;" ::: "memory"); }
 
 // Index k of an axis of n nodes: wrapped on a periodic axis, the nearest node
 // on a walled one.
@@ -45,20 +43,6 @@ __device__ __forceinline__ void ring_site(int q, int &c, int &r)
         r += H;
         if (c >= H / 2) c += kTP;
     }
-}
-
-// A launch of kNT threads per block that may start while the previous one on the
-// stream still runs; its blocks call chain_wait before they touch its results.
-inline void chained_launch(cudaLaunchConfig_t &cfg, cudaLaunchAttribute &at, dim3 grid, size_t smem, cudaStream_t s)
-{
-    cfg.gridDim = grid;
-    cfg.blockDim = dim3(kNT);
-    cfg.dynamicSmemBytes = smem;
-    cfg.stream = s;
-    at.id = cudaLaunchAttributeProgrammaticStreamSerialization;
-    at.val.programmaticStreamSerializationAllowed = 1;
-    cfg.attrs = &at;
-    cfg.numAttrs = 1;
 }
 
 }  // namespace

@@ -149,7 +149,7 @@ def test_tile_step_is_the_automatic_choice_on_small_and_medium_grids():
     assert kernel(896, 896) == kernel(300, 33) == "fused-warp"
     assert kernel(1096, 1092, has_force=True) == "fused-tile" and kernel(1100, 1096, has_force=True) == "fused-warp"
     assert kernel(1095, 1095) == "fused-tile" and kernel(1097, 1097) == "fused"
-    assert kernel(1161, 1161, walls=True) == "fused-tile" and kernel(1163, 1163, walls=True) == "fused-warp"
+    assert kernel(1117, 1117, walls=True) == "fused-tile" and kernel(1119, 1119, walls=True) == "fused-warp"
     assert kernel(60, 45000, walls=True) == "fused-tile"
     assert kernel(64, 64, variant="warp") == kernel(64, 64, rows_per_cta=4) == kernel(64, 64, path="fused") == "fused-warp"
     assert kernel(33, 33, walls=True, path="fused") == "fused-walls"
