@@ -94,7 +94,7 @@ int choose_path(const fdlbm_grid *g, const fdlbm_opts *o)
 // is taken, and for FP64 grids unless a tile height or a kernel is asked for.
 // FP64 is bound by the FP64 units, and the split step does no node's work
 // twice (us per step on GB300, sweep or staged kernels -> split: 64^2 periodic
-// 59.6 -> 11.6, 257^2 cavity 81 -> 35, 1024^2 periodic 718 -> 431); in FP32 the
+// 59.6 -> 7.1, 257^2 cavity 81 -> 35, 1024^2 periodic 718 -> 431); in FP32 the
 // sweeps move a third of its bytes (2048^2: 70 against 205).
 bool use_split(const fdlbm_opts *o, int path)
 {

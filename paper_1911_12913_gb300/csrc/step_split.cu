@@ -28,6 +28,7 @@
 // 35.1 (five staged launches with a thread per wall node 81).
 #include <algorithm>
 #include <cmath>
+#include <type_traits>
 #include <vector>
 
 #include "chain.cuh"
@@ -43,6 +44,10 @@ namespace {
 // 35.1 us per step, 45.5 in blocks of 128, 1024^2: the same either way).
 template <class R>
 constexpr int kThreads = sizeof(R) == 8 ? 32 : 128;
+
+// FP64 wall nodes take four threads each (Quad, below).
+template <class R>
+constexpr bool kQuadWalls = sizeof(R) == 8;
 
 // The launches of a call are chained (chain.cuh).  Letting the next one's blocks
 // in at the start of the kernel instead of after a warp's arithmetic made them
@@ -169,12 +174,14 @@ struct Site {
 // Node coordinates of this thread.  Wall nodes come first, in blocks of their
 // own (a warp that holds both kinds would run Eq. 3.10 for its interior lanes
 // too); then the rectangle, linear over strips of `strip` columns, so that
-// every warp is full on any width.  False past the end.
-template <class R, bool WALLS>
+// every warp is full on any width.  LANES threads share a node.  False past the
+// end.
+template <class R, bool WALLS, int LANES = 1>
 __device__ __forceinline__ bool my_node(const SplitArgs<R> &a, int &x, int &y)
 {
+    const int per_block = blockDim.x / LANES, t = threadIdx.x / LANES;
     if (WALLS && blockIdx.x < a.wall_blocks) {
-        const int k = blockIdx.x * blockDim.x + threadIdx.x;
+        const int k = blockIdx.x * per_block + t;
         const int rows = a.wy ? 2 * a.nx : 0;  // S and N rows, corners included
         if (k < rows) {
             x = k < a.nx ? k : k - a.nx;
@@ -188,7 +195,7 @@ __device__ __forceinline__ bool my_node(const SplitArgs<R> &a, int &x, int &y)
     }
     const int b = blockIdx.x - (WALLS ? a.wall_blocks : 0);
     const int strip = b / a.strip_blocks;
-    const unsigned k = (b - strip * a.strip_blocks) * blockDim.x + threadIdx.x;
+    const unsigned k = (b - strip * a.strip_blocks) * per_block + t;
     const int xs = strip * a.strip;
     const unsigned w = min(a.strip, a.w - xs);
     const unsigned row = k / w;
@@ -332,6 +339,222 @@ __device__ __forceinline__ void load_force(const SplitArgs<R> &a, int x, int y, 
     }
 }
 
+// Four threads per node, for grids and wall nodes that leave schedulers idle: a
+// node's chain of FP64 instructions (48 in the star kernel, 55 in the update,
+// against 104 and 123) is what such a launch waits for.  Thread q of a node takes
+// the axis velocity 1 + q and the diagonal one 5 + q, whose differences run along
+// the same half axes; the moments are summed over the four by shuffles, and the
+// rest population is everybody's.  Every thread of the warp takes part in the
+// shuffles: those past the last node work on a copy of the first.  (129^2 cavity,
+// whose wall nodes alone are split: 20.9 -> 14.2 us per step; 64^2 periodic 11.6 ->
+// 7.1.)
+template <class R, bool FORCE>
+struct Quad {
+    const SplitArgs<R> &a;
+    const int q;
+    const R ax, ay, dx, dy;  // velocities
+    Taps<R> wx, wy;
+    int o0, x[3], y[3];      // offsets at k, and at k + s, k - s, k - 2s in x and in y
+    R drho, jx, jy, rm, inv, h45, base;
+
+    __device__ __forceinline__ explicit Quad(const SplitArgs<R> &a_)
+        : a(a_), q(threadIdx.x & 3), ax(R(q == 0) - R(q == 2)), ay(R(q == 1) - R(q == 3)),
+          dx(q == 0 || q == 3 ? R(1) : R(-1)), dy(q < 2 ? R(1) : R(-1))
+    {
+    }
+
+    __device__ __forceinline__ static int index(int k, int n, bool wall)
+    {
+        return wall ? min(max(k, 0), n - 1) : k < 0 ? k + n : (k >= n ? k - n : k);
+    }
+
+    __device__ __forceinline__ void set(int xc, int yc)
+    {
+        const int sx = q == 0 || q == 3 ? 1 : -1, sy = q < 2 ? 1 : -1;
+        const int at[3] = {1, -1, -2};
+        const int row = yc * a.pitch;
+        o0 = row + xc;
+#pragma unroll
+        for (int k = 0; k < 3; ++k) {
+            x[k] = row + index(xc + at[k] * sx, a.nx, a.wx);
+            y[k] = index(yc + at[k] * sy, a.ny, a.wy) * a.pitch + xc;
+        }
+        wx = load_taps(a.tx + 8 * xc + (sx > 0 ? 0 : 4));
+        wy = load_taps(a.ty + 8 * yc + (sy > 0 ? 0 : 4));
+    }
+
+    // acc plus the weighted taps of the axis and of the diagonal population
+    __device__ __forceinline__ R axis(const R *f, R acc) const
+    {
+        const bool h = !(q & 1);
+        acc = fma(h ? wx.c : wy.c, f[o0], acc);
+        acc = fma(h ? wx.m1 : wy.m1, f[h ? x[0] : y[0]], acc);
+        acc = fma(h ? wx.p1 : wy.p1, f[h ? x[1] : y[1]], acc);
+        return fma(h ? wx.p2 : wy.p2, f[h ? x[2] : y[2]], acc);
+    }
+    __device__ __forceinline__ R diagonal(const R *f, R acc) const
+    {
+        acc = fma(wx.c + wy.c, f[o0], acc);
+        acc = fma(wx.m1, f[x[0]], acc);
+        acc = fma(wy.m1, f[y[0]], acc);
+        acc = fma(wx.p1, f[x[1]], acc);
+        acc = fma(wy.p1, f[y[1]], acc);
+        acc = fma(wx.p2, f[x[2]], acc);
+        return fma(wy.p2, f[y[2]], acc);
+    }
+
+    __device__ __forceinline__ static R sum4(R v)
+    {
+        v += __shfl_xor_sync(0xffffffffu, v, 1);
+        return v + __shfl_xor_sync(0xffffffffu, v, 2);
+    }
+
+    // Eq. 3.3 (force shift `shift`) and the common terms of Eq. 3.2
+    __device__ __forceinline__ void macro(R g0, R ga, R gd, R Fx, R Fy, R shift)
+    {
+        drho = sum4(ga + gd) + g0;
+        jx = sum4(fma(dx, gd, ax * ga));
+        jy = sum4(fma(dy, gd, ay * ga));
+        rm = macro_density(a.c, drho);
+        if (FORCE) {
+            jx += shift * rm * Fx;
+            jy += shift * rm * Fy;
+        }
+        inv = node_reciprocal(rm);
+        const R jj = jx * jx + jy * jy;
+        h45 = R(4.5) * inv;
+        base = fma(jj, R(-1.5) * inv, drho);
+    }
+    __device__ __forceinline__ void equilibrium(R &e0, R &ea, R &ed) const
+    {
+        const R ja = fma(ax, jx, ay * jy), jd = fma(dx, jx, dy * jy);
+        e0 = wq<R>(0) * base;
+        ea = fma(LinearCoef<R>::c1, ja, wq<R>(1) * fma(ja * ja, h45, base));
+        ed = fma(LinearCoef<R>::c2, jd, wq<R>(5) * fma(jd * jd, h45, base));
+    }
+    // Eq. 3.12 at the equilibrium (e0, ea, ed)
+    __device__ __forceinline__ void force_term(R e0, R ea, R ed, R Fx, R Fy, R &f0, R &fa, R &fd) const
+    {
+        const R nuF = -(jx * Fx + jy * Fy) * inv, r0 = a.c.rho0 - force_dshift(a.c, drho);
+        f0 = R(3) * nuF * fma(wq<R>(0), r0, e0);
+        fa = R(3) * (nuF + fma(ax, Fx, ay * Fy)) * fma(wq<R>(1), r0, ea);
+        fd = R(3) * (nuF + fma(dx, Fx, dy * Fy)) * fma(wq<R>(5), r0, ed);
+    }
+    // Eq. 3.10 from x_j's values
+    __device__ __forceinline__ void extrapolate(int side, R Fx, R Fy, R shift, R &g0, R &ga, R &gd)
+    {
+        R u, v, e0, ea, ed;
+        wall_velocity(a, side, u, v);
+        macro(g0, ga, gd, Fx, Fy, shift);
+        equilibrium(e0, ea, ed);
+        const R ua = fma(ax, u, ay * v), ud = fma(dx, u, dy * v), uu = R(1.5) * (u * u + v * v);
+        g0 = wq<R>(0) * (drho - rm * uu) + (g0 - e0);
+        ga = wq<R>(1) * (drho + rm * (ua * (R(3) + R(4.5) * ua) - uu)) + (ga - ea);
+        gd = wq<R>(5) * (drho + rm * (ud * (R(3) + R(4.5) * ud) - uu)) + (gd - ed);
+    }
+};
+
+template <class R, bool FORCE, bool WALLS>
+__device__ __forceinline__ void star_quad(const SplitArgs<R> &a)
+{
+    int x, y;
+    const bool valid = my_node<R, WALLS, 4>(a, x, y);
+    const bool walls = WALLS && blockIdx.x < a.wall_blocks;
+    if (!valid) {
+        x = walls ? 0 : a.x0;
+        y = walls ? 0 : a.y0;
+    }
+    int jx = x, jy = y, side = -1;
+    if (WALLS) side = wall_side(a, x, y, jx, jy);  // a wall for the whole block, or for none of it
+    Quad<R, FORCE> n(a);
+    n.set(jx, jy);
+    R Fx, Fy;
+    load_force<R, FORCE>(a, jx, jy, Fx, Fy);
+    chain_wait();
+    const size_t pa = (1 + n.q) * a.plane, pd = (5 + n.q) * a.plane;
+    R g0 = a.P[n.o0], ga = n.axis(a.P + pa, a.P[pa + n.o0]), gd = n.diagonal(a.P + pd, a.P[pd + n.o0]);
+    n.macro(g0, ga, gd, Fx, Fy, a.c.half_h);
+    R e0, ea, ed;
+    n.equilibrium(e0, ea, ed);
+    const R b = a.c.b_star;
+    g0 = fma(b, e0 - g0, g0);
+    ga = fma(b, ea - ga, ga);
+    gd = fma(b, ed - gd, gd);
+    if (FORCE) {
+        R f0, fa, fd;
+        n.force_term(e0, ea, ed, Fx, Fy, f0, fa, fd);
+        g0 = fma(a.c.c_star, f0, g0);
+        ga = fma(a.c.c_star, fa, ga);
+        gd = fma(a.c.c_star, fd, gd);
+    }
+    if (WALLS && walls) n.extrapolate(side, R(0), R(0), R(0), g0, ga, gd);
+    chain_next();
+    if (!valid) return;
+    const size_t o = (size_t)y * a.pitch + x;
+    a.S[pa + o] = ga;
+    a.S[pd + o] = gd;
+}
+
+template <class R, bool FORCE, bool WALLS, bool LAST>
+__device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
+{
+    int x, y;
+    const bool valid = my_node<R, WALLS, 4>(a, x, y);
+    const bool walls = WALLS && blockIdx.x < a.wall_blocks;
+    if (!valid) {
+        x = walls ? 0 : a.x0;
+        y = walls ? 0 : a.y0;
+    }
+    int jx = x, jy = y, side = -1;
+    if (WALLS) side = wall_side(a, x, y, jx, jy);
+    Quad<R, FORCE> n(a);
+    n.set(jx, jy);
+    chain_wait();
+    const size_t pa = (1 + n.q) * a.plane, pd = (5 + n.q) * a.plane;
+    R g0 = a.Qin[n.o0], ga = n.axis(a.S + pa, a.Qin[pa + n.o0]), gd = n.diagonal(a.S + pd, a.Qin[pd + n.o0]);
+    R Fx, Fy;
+    if (WALLS && walls) {
+        load_force<R, FORCE>(a, jx, jy, Fx, Fy);
+        n.extrapolate(side, Fx, Fy, a.c.half_dt, g0, ga, gd);
+    }
+    const size_t o = (size_t)y * a.pitch + x;
+    if (LAST) {
+        if (!valid) return;
+        if (n.q == 0) a.Qout[o] = g0;
+        a.Qout[pa + o] = ga;
+        a.Qout[pd + o] = gd;
+        return;
+    }
+    load_force<R, FORCE>(a, x, y, Fx, Fy);
+    n.macro(g0, ga, gd, Fx, Fy, a.c.half_dt);
+    R e0, ea, ed, f0 = R(0), fa = R(0), fd = R(0);
+    n.equilibrium(e0, ea, ed);
+    if (FORCE) n.force_term(e0, ea, ed, Fx, Fy, f0, fa, fd);
+    auto relax = [&](R g, R e, R f, R &P, R &Q) {
+        const R neq = e - g;
+        P = fma(a.c.b_bar, neq, g);
+        Q = fma(a.c.b_til, neq, g);
+        if (FORCE) {
+            P = fma(a.c.c_bar, f, P);
+            Q = fma(a.c.c_til, f, Q);
+        }
+    };
+    R P0, Q0, Pa, Qa, Pd, Qd;
+    relax(g0, e0, f0, P0, Q0);
+    relax(ga, ea, fa, Pa, Qa);
+    relax(gd, ed, fd, Pd, Qd);
+    chain_next();
+    if (!valid) return;
+    if (n.q == 0) {
+        a.P[o] = P0;
+        a.Qout[o] = Q0;
+    }
+    a.P[pa + o] = Pa;
+    a.P[pd + o] = Pd;
+    a.Qout[pa + o] = Qa;
+    a.Qout[pd + o] = Qd;
+}
+
 template <class R, bool FORCE>
 __global__ void __launch_bounds__(kThreads<R>) k_split_prepare(const SplitArgs<R> a)
 {
@@ -351,9 +574,15 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_prepare(const SplitArgs<R
     }
 }
 
-template <class R, bool FORCE, bool WALLS>
+// QUAD: four threads per node for every node; else for the wall nodes of an FP64
+// grid.
+template <class R, bool FORCE, bool WALLS, bool QUAD>
 __global__ void __launch_bounds__(kThreads<R>) k_split_star(const SplitArgs<R> a)
 {
+    if (QUAD || (WALLS && kQuadWalls<R> && blockIdx.x < a.wall_blocks)) {
+        star_quad<R, FORCE, WALLS>(a);
+        return;
+    }
     int x, y;
     if (!my_node<R, WALLS>(a, x, y)) return;
     int jx = x, jy = y, side = -1;
@@ -384,9 +613,13 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_star(const SplitArgs<R> a
     for (int i = 1; i < 9; ++i) a.S[i * a.plane + o] = st[i];
 }
 
-template <class R, bool FORCE, bool WALLS, bool LAST>
+template <class R, bool FORCE, bool WALLS, bool QUAD, bool LAST>
 __global__ void __launch_bounds__(kThreads<R>) k_split_update(const SplitArgs<R> a)
 {
+    if (QUAD || (WALLS && kQuadWalls<R> && blockIdx.x < a.wall_blocks)) {
+        update_quad<R, FORCE, WALLS, LAST>(a);
+        return;
+    }
     int x, y;
     if (!my_node<R, WALLS>(a, x, y)) return;
     int jx = x, jy = y, side = -1;
@@ -429,11 +662,12 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_update(const SplitArgs<R>
 }
 
 // One launch over all nodes; split_walls: the wall nodes in blocks of their
-// own.  chained: scheduled while the previous launch of the chain still runs.
+// own.  lanes: threads per node (1 or 4).  chained: scheduled while the previous launch of the chain still runs.
 template <class R, class K>
-cudaError_t launch(K kernel, SplitArgs<R> a, bool split_walls, bool chained, cudaStream_t s)
+cudaError_t launch(K kernel, SplitArgs<R> a, int lanes, bool split_walls, bool chained, cudaStream_t s)
 {
     constexpr int nt = kThreads<R>;
+    const int nodes = nt / lanes, wall_nodes = kQuadWalls<R> ? nt / 4 : nodes;  // per block
     const int wx = split_walls && a.wx, wy = split_walls && a.wy;
     a.x0 = wx;
     a.y0 = wy;
@@ -441,35 +675,35 @@ cudaError_t launch(K kernel, SplitArgs<R> a, bool split_walls, bool chained, cud
     a.h = a.ny - 2 * wy;
     const int strips = (a.w + 63) / 64;
     a.strip = (a.w + strips - 1) / strips;
-    a.strip_blocks = (int)(((long long)a.strip * a.h + nt - 1) / nt);
+    a.strip_blocks = (int)(((long long)a.strip * a.h + nodes - 1) / nodes);
     const long long walls = (wy ? 2ll * a.nx : 0) + (wx ? 2ll * a.h : 0);
-    a.wall_blocks = (int)((walls + nt - 1) / nt);
+    a.wall_blocks = (int)((walls + wall_nodes - 1) / wall_nodes);
     const dim3 grid((unsigned)(a.wall_blocks + a.strip_blocks * ((a.w + a.strip - 1) / a.strip)));
     if (chained) return chained_launch(kernel, grid, nt, 0, s, a);
     kernel<<<grid, nt, 0, s>>>(a);
     return cudaGetLastError();
 }
 
-template <class R, bool FORCE, bool WALLS>
+template <class R, bool FORCE, bool WALLS, bool QUAD>
 cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStream_t s)
 {
     const R *bx = tabs, *by = tabs + 8 * (size_t)a.nx;                     // stage B (scale -h m)
     const R *cxs = by + 8 * (size_t)a.ny, *cys = cxs + 8 * (size_t)a.nx;   // stage C (scale -dt m)
     R *q[2] = {Q0, Q1};
     a.Qout = q[0];
-    cudaError_t e = launch<R>(k_split_prepare<R, FORCE>, a, false, false, s);
+    cudaError_t e = launch<R>(k_split_prepare<R, FORCE>, a, 1, false, false, s);
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         const bool last = k + 1 == nsteps;
         a.tx = bx;
         a.ty = by;
-        e = launch<R>(k_split_star<R, FORCE, WALLS>, a, WALLS, true, s);
+        e = launch<R>(k_split_star<R, FORCE, WALLS, QUAD>, a, QUAD ? 4 : 1, WALLS, true, s);
         if (e != cudaSuccess) break;
         a.tx = cxs;
         a.ty = cys;
         a.Qin = q[k & 1];
         a.Qout = last ? a.P : q[(k + 1) & 1];
-        e = last ? launch<R>(k_split_update<R, FORCE, WALLS, true>, a, WALLS, true, s)
-                 : launch<R>(k_split_update<R, FORCE, WALLS, false>, a, WALLS, true, s);
+        e = last ? launch<R>(k_split_update<R, FORCE, WALLS, QUAD, true>, a, QUAD ? 4 : 1, WALLS, true, s)
+                 : launch<R>(k_split_update<R, FORCE, WALLS, QUAD, false>, a, QUAD ? 4 : 1, WALLS, true, s);
     }
     return e;
 }
@@ -533,6 +767,11 @@ template std::vector<double> make_split_tables<double>(const std::vector<double>
                                                        bool, double, double, double);
 
 // nsteps steps of the state in s.gin, in place.
+// Grids of at most so many nodes take four threads per node throughout: up to two
+// such warps per scheduler of 152 SMs on a periodic grid, one on a walled one
+// (us per step, four threads against one: 24^2 6.4 / 11.7, 64^2 7.1 / 11.6, 96^2
+// 10.9 / 12.5, 120^2 15.1 / 13.0; walled 65^2 10.6 / 13.2, 97^2 14.2 / 13.6).
+constexpr long long kQuadNodes = 9728, kQuadWalledNodes = 4864;
 template <class R>
 cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream)
 {
@@ -556,11 +795,21 @@ cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, in
     a.w_star[2] = s.c.b_star * wq<R>(5);
     a.l_star[0] = s.c.b_star * LinearCoef<R>::c1;
     a.l_star[1] = s.c.b_star * LinearCoef<R>::c2;
-    if (a.wx || a.wy)
-        return s.force ? run<R, true, true>(a, Q0, Q1, tables, nsteps, stream)
-                       : run<R, false, true>(a, Q0, Q1, tables, nsteps, stream);
-    return s.force ? run<R, true, false>(a, Q0, Q0, tables, nsteps, stream)
-                   : run<R, false, false>(a, Q0, Q0, tables, nsteps, stream);
+    const bool walls = a.wx || a.wy;
+    auto go = [&](auto force, auto wl, auto quad) {
+        constexpr bool F = decltype(force)::value, W = decltype(wl)::value, Q = decltype(quad)::value;
+        return run<R, F, W, Q>(a, Q0, Q1, tables, nsteps, stream);
+    };
+    auto pick = [&](auto quad) {
+        const std::true_type y{};
+        const std::false_type n{};
+        if (walls) return s.force ? go(y, y, quad) : go(n, y, quad);
+        return s.force ? go(y, n, quad) : go(n, n, quad);
+    };
+    if constexpr (sizeof(R) == 8) {
+        if ((long long)a.nx * a.ny <= (walls ? kQuadWalledNodes : kQuadNodes)) return pick(std::true_type{});
+    }
+    return pick(std::false_type{});
 }
 template cudaError_t launch_split<float>(const StepArgs<float> &, float *, float *, const float *, int, cudaStream_t);
 template cudaError_t launch_split<double>(const StepArgs<double> &, double *, double *, const double *, int,

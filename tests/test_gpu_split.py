@@ -1,5 +1,6 @@
 """The step in two launches (step_split.cu), which FP64 grids take by default
-and path="staged" in both precisions, against the oracle: strips of one column
+and path="staged" in both precisions, against the oracle (four threads per node on
+small FP64 grids and at FP64 wall nodes): strips of one column
 to several, partial last warps and strips, grids of three nodes per axis, every
 boundary combination with moving walls, random metrics, a force field, the
 incompressible equilibrium, A = 0, direct launches and a replayed graph."""
@@ -41,7 +42,13 @@ def _axis(kind, n, seed, length):
     ("wall", "wall", 131, 9, {"force": True}), ("periodic", "wall", 130, 34, {"force": True, "graph": 2}),
     ("wall", "periodic", 67, 40, {"eq": "incompressible", "force": True}),
     ("periodic", "periodic", 96, 40, {"eq": "incompressible"}), ("periodic", "wall", 64, 20, {"A": 0.0}),
-    ("wall", "wall", 257, 40, {}), ("periodic", "periodic", 200, 129, {}),
+    # FP64 grids past the sizes that take four threads per node throughout
+    ("wall", "wall", 257, 40, {}), ("periodic", "periodic", 200, 129, {}), ("periodic", "periodic", 160, 64, {"force": True}),
+    ("wall", "wall", 131, 80, {"force": True, "graph": 2}), ("periodic", "wall", 150, 70, {"force": True}),
+    ("wall", "periodic", 140, 90, {"eq": "incompressible", "force": True}), ("wall", "wall", 99, 98, {"A": 0.0}),
+    # and on both sides of those lines
+    ("periodic", "periodic", 128, 76, {}), ("periodic", "periodic", 139, 70, {}), ("wall", "wall", 76, 64, {}),
+    ("wall", "wall", 65, 75, {}),
 ])
 def test_split_step_matches_oracle(precision, x, y, nx, ny, more):
     xa, ya = _axis(x, nx, 31, 1.0), _axis(y, ny, 32, 0.8)
