@@ -129,11 +129,12 @@ typedef struct {
     int has_force;            /* 1: reserve a body-acceleration field (fdlbm_set_force), Eq. 3.12 */
     int path;                 /* FDLBM_PATH_AUTO: the fused path for both schemes on periodic
                                  grids and on walled grids in FP32; the staged path for
-                                 walled grids in FP64.  T2S2-FDLBM1 takes the split step (two
-                                 launches per step and one more per call, one node per
-                                 thread, no halo recomputed) on the staged path, and in FP64
-                                 on either one unless rows_per_cta or variant is set: FP64
-                                 is bound by the FP64 units */
+                                 walled grids in FP64.  T2S2-FDLBM1 in FP64 takes the split
+                                 step (two launches per step and one more per call, one node
+                                 per thread, no halo recomputed) on the staged path, and on
+                                 the fused one unless rows_per_cta or variant is set or the
+                                 grid has more than 2^28 nodes: FP64 is bound by the FP64
+                                 units */
     int rows_per_cta;         /* fused kernel tile height; 0 = automatic */
     int variant;              /* FDLBM_VARIANT_*; WARP where it does not apply -> EUNSUPPORTED */
     int scheme;               /* FDLBM_SCHEME_T2S2_1 (default) or FDLBM_SCHEME_T2S2_2 */
@@ -243,7 +244,9 @@ int fdlbm_kernels_per_step(fdlbm_t h);   /* kernel launches fdlbm_step makes per
  * column), the end of the columns the tile stores, y0, y1 (rows [y0, y1)).
  * The interior covers the nodes at least 4 from every wall whose tiles load
  * nothing outside the grid (Eq. 3.10 and the central differences next to a
- * wall reach no further), the frame the rest.  Host only, no device work:
+ * wall reach no further), the frame the rest (with variant AUTO the frame of a
+ * T2S2_1 grid runs on the tiles of the tile kernel instead, which store the
+ * same nodes).  Host only, no device work:
  * *count receives the number of tiles and at most cap are written to tiles.
  * EINVAL for bad arguments, EUNSUPPORTED where the warp-tile kernel does not
  * apply. */

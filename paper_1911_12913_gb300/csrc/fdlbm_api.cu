@@ -90,17 +90,19 @@ int choose_path(const fdlbm_grid *g, const fdlbm_opts *o)
     return can_fuse ? FDLBM_PATH_FUSED : FDLBM_PATH_STAGED;
 }
 
-// T2S2-FDLBM1 in two launches per step (step_split.cu) where the staged path
-// is taken, and for FP64 grids unless a tile height or a kernel is asked for.
+// FP64 T2S2-FDLBM1 in two launches per step (step_split.cu) where the staged path
+// is taken, and on other grids unless a tile height or a kernel is asked for.
 // FP64 is bound by the FP64 units, and the split step does no node's work
 // twice (us per step on GB300, sweep or staged kernels -> split: 64^2 periodic
 // 59.6 -> 7.1, 257^2 cavity 81 -> 35, 1024^2 periodic 718 -> 431); in FP32 the
-// sweeps move a third of its bytes (2048^2: 70 against 205).
-bool use_split(const fdlbm_opts *o, int path)
+// sweeps move a third of its bytes (2048^2: 70 against 205).  Periodic grids past
+// 2^28 nodes (two states of 39 GB) keep the sweep, which needs no scratch field.
+bool use_split(const fdlbm_grid *g, const fdlbm_opts *o, int path)
 {
-    if (o->scheme != FDLBM_SCHEME_T2S2_1) return false;
+    if (o->scheme != FDLBM_SCHEME_T2S2_1 || o->precision != FDLBM_FP64) return false;
     if (path == FDLBM_PATH_STAGED) return true;
-    return o->precision == FDLBM_FP64 && o->path == FDLBM_PATH_AUTO && o->variant == FDLBM_VARIANT_AUTO &&
+    if ((long long)g->nx * g->ny > (1ll << 28)) return false;
+    return o->path == FDLBM_PATH_AUTO && o->variant == FDLBM_VARIANT_AUTO &&
            o->rows_per_cta == 0;
 }
 
@@ -149,7 +151,7 @@ bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
 int scratch_fields(const fdlbm_grid *g, const fdlbm_opts *o, int path, bool force_staged)
 {
     if (force_staged || path == FDLBM_PATH_STAGED || o->adjoint) return 3;
-    if (use_split(o, path)) return walled(g) ? 2 : 1;
+    if (use_split(g, o, path)) return walled(g) ? 2 : 1;
     return 0;
 }
 
@@ -223,20 +225,13 @@ StepArgs<R> step_args(fdlbm_ctx *h)
     return a;
 }
 
-template <class R>
-cudaError_t launch_split_steps(fdlbm_ctx *h, int n, cudaStream_t s)
-{
-    const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
-    R *q0 = reinterpret_cast<R *>(h->ws + h->lay.Q);
-    R *q1 = walls ? reinterpret_cast<R *>(h->ws + h->lay.P) : q0;
-    return launch_split<R>(step_args<R>(h), q0, q1, reinterpret_cast<const R *>(h->ws + h->lay.split), n, s);
-}
-
 // n steps of the split kernels (the state stays in state[cur]), on stream s.
 cudaError_t launch_split_steps(fdlbm_ctx *h, int n, cudaStream_t s)
 {
-    return h->precision == FDLBM_FP32_DEV ? launch_split_steps<float>(h, n, s)
-                                          : launch_split_steps<double>(h, n, s);
+    const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
+    double *q0 = reinterpret_cast<double *>(h->ws + h->lay.Q);
+    double *q1 = walls ? reinterpret_cast<double *>(h->ws + h->lay.P) : q0;
+    return launch_split(step_args<double>(h), q0, q1, reinterpret_cast<const double *>(h->ws + h->lay.split), n, s);
 }
 
 // One step of whichever kernel the handle uses, reading state[cur], on stream s.
@@ -492,7 +487,7 @@ Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, int 
     if (scratch > 0) L.Q = take(9 * plane * rs);
     if (scratch > 1) L.P = take(9 * plane * rs);
     if (scratch > 2) L.S = take(9 * plane * rs);
-    if (split) L.split = take(split_table_bytes(nx, ny, rs));
+    if (split) L.split = take(split_table_bytes(nx, ny));
     L.uprev = take(2 * (size_t)nx * ny * sizeof(double));
     L.nblocks_red = kRedBlocks;
     L.partials = take((size_t)kRedBlocks * 3 * sizeof(double));
@@ -591,7 +586,7 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->stream = static_cast<cudaStream_t>(o.stream);
     h->adjoint = o.adjoint != 0;
     h->graph_steps = o.graph_steps > 0 ? o.graph_steps + (o.graph_steps & 1) : 0;
-    h->split = !force_staged && use_split(&o, path);
+    h->split = !force_staged && use_split(g, &o, path);
     h->tile = !force_staged && use_tile(g, &o, path);
     h->tile_frame = !force_staged && walled(g) && s1 && o.variant == FDLBM_VARIANT_AUTO;
     h->lay = make_layout(h->nx, h->ny, h->pitch, h->precision, h->has_force,
@@ -601,18 +596,11 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     return FDLBM_OK;
 }
 
-template <class R>
-static cudaError_t upload_split_tables_t(fdlbm_ctx *h, const std::vector<double> &mx, const std::vector<double> &my)
-{
-    const std::vector<R> t = make_split_tables<R>(mx, my, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, h->beta,
-                                                  h->A * h->dt, h->dt);
-    return cudaMemcpy(h->ws + h->lay.split, t.data(), t.size() * sizeof(R), cudaMemcpyHostToDevice);
-}
-
 static cudaError_t upload_split_tables(fdlbm_ctx *h, const std::vector<double> &mx, const std::vector<double> &my)
 {
-    return h->precision == FDLBM_FP32_DEV ? upload_split_tables_t<float>(h, mx, my)
-                                          : upload_split_tables_t<double>(h, mx, my);
+    const std::vector<double> t = make_split_tables(mx, my, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, h->beta,
+                                                    h->A * h->dt, h->dt);
+    return cudaMemcpy(h->ws + h->lay.split, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice);
 }
 
 // Zero the state (fluid at rest) and the force, clear the error flag, upload
@@ -687,7 +675,7 @@ size_t fdlbm_workspace_bytes(const fdlbm_grid *g, const fdlbm_opts *opts)
     const int path = choose_path(g, &o);
     if (path < 0) return 0;
     return make_layout(g->nx, g->ny, pitch_of(g->nx), o.precision, o.has_force,
-                       scratch_fields(g, &o, path, false), use_split(&o, path))
+                       scratch_fields(g, &o, path, false), use_split(g, &o, path))
         .total;
 }
 

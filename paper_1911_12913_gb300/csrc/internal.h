@@ -180,14 +180,13 @@ cudaError_t launch_fused_walls(const StepArgs<R> &a, cudaStream_t s);
 template <class R>
 int fused_walls_blocks_per_sm();
 int fused_tile_width_walls();
-// step_split.cu (two launches per step, one node per thread; the state in
+// step_split.cu (FP64, two launches per step, one node per thread; the state in
 // s.gin is advanced in place, s.gout is scratch)
-size_t split_table_bytes(int nx, int ny, size_t real_size);
-template <class R>
-std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
-                                 double beta, double h, double dt);
-template <class R>
-cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream);
+size_t split_table_bytes(int nx, int ny);
+std::vector<double> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
+                                      double beta, double h, double dt);
+cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, int nsteps,
+                         cudaStream_t stream);
 // step_tile.cu (FP32 T2S2-FDLBM1, one launch per step, a tile per block)
 void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty);
 cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s);

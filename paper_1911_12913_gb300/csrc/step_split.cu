@@ -1,4 +1,4 @@
-// The T2S2-FDLBM1 step in two launches per step, one node per thread, for any
+// The FP64 T2S2-FDLBM1 step in two launches per step, one node per thread, for any
 // boundary combination: each quantity of Sec. 2D is formed once per node, with
 // no halo recomputed.
 //
@@ -18,14 +18,14 @@
 // a wall, where the second-order upwind tap would leave the domain, the entry
 // of that sign holds the central difference.
 //
-// What bounds it.  FP64: the FP64 units, 227 FP64 instructions per node (prepare
+// What bounds it: the FP64 units, 227 FP64 instructions per node (prepare
 // 79, star 104, update 44): 1024^2 periodic 431 us per step, 0.87 of the rate at
 // which a warp's FP64 instruction takes 64 cycles of its scheduler; the 576
 // bytes per node that pass between the launches are hidden behind them.  The
 // sweep it replaced there recomputed 8 halo rows and columns per tile and spent
-// 281 instructions per node: 718 us.  Small grids wait for launches and for one
-// warp's chain of instructions: 64^2 11.6 us per step (sweep 59.6), 257^2 cavity
-// 35.1 (five staged launches with a thread per wall node 81).
+// 239 instructions per node: 718 us.  Small grids wait for launches and for one
+// warp's chain of instructions: 64^2 7.1 us per step (sweep 59.6), 257^2 cavity
+// 34.6 (five staged launches with a thread per wall node 81).
 #include <algorithm>
 #include <cmath>
 #include <type_traits>
@@ -38,16 +38,11 @@
 namespace fdlbm {
 namespace {
 
-// Threads per block.  FP64: one warp.  A warp's FP64 instruction holds its
+// Threads per block: one warp.  A warp's FP64 instruction holds its
 // scheduler's FP64 unit for 64 cycles, so a launch lasts as long as the
 // scheduler with the most warps; single warps spread most evenly (257^2 cavity:
 // 35.1 us per step, 45.5 in blocks of 128, 1024^2: the same either way).
-template <class R>
-constexpr int kThreads = sizeof(R) == 8 ? 32 : 128;
-
-// FP64 wall nodes take four threads each (Quad, below).
-template <class R>
-constexpr bool kQuadWalls = sizeof(R) == 8;
+constexpr int kThreads = 32;
 
 // The launches of a call are chained (chain.cuh).  Letting the next one's blocks
 // in at the start of the kernel instead of after a warp's arithmetic made them
@@ -80,22 +75,9 @@ struct Taps {
 template <class R>
 __device__ __forceinline__ Taps<R> load_taps(const R *t)
 {
-    Taps<R> w;
-    if constexpr (sizeof(R) == 4) {
-        const float4 v = __ldg(reinterpret_cast<const float4 *>(t));
-        w.m1 = v.x;
-        w.c = v.y;
-        w.p1 = v.z;
-        w.p2 = v.w;
-    } else {
-        const double2 u = __ldg(reinterpret_cast<const double2 *>(t));
-        const double2 v = __ldg(reinterpret_cast<const double2 *>(t) + 1);
-        w.m1 = u.x;
-        w.c = u.y;
-        w.p1 = v.x;
-        w.p2 = v.y;
-    }
-    return w;
+    const double2 u = __ldg(reinterpret_cast<const double2 *>(t));
+    const double2 v = __ldg(reinterpret_cast<const double2 *>(t) + 1);
+    return {u.x, u.y, v.x, v.y};
 }
 
 // A node, its neighbours (wrapped on a periodic axis; on a walled axis clamped,
@@ -127,47 +109,25 @@ struct Site {
     __device__ __forceinline__ R advance(const R *f, int i, R v0, R acc) const
     {
         const int r0 = y[2];
-        if constexpr (sizeof(R) == 8) {
-            // FP64: one multiply-add per tap, the centre weights of a diagonal merged
-            if (cx(i) != 0 && cy(i) != 0) acc = fma((cx(i) > 0 ? xp.c : xn.c) + (cy(i) > 0 ? yp.c : yn.c), v0, acc);
-            else if (cx(i) != 0) acc = fma(cx(i) > 0 ? xp.c : xn.c, v0, acc);
-            else acc = fma(cy(i) > 0 ? yp.c : yn.c, v0, acc);
-            if (cx(i) != 0) {
-                const Taps<R> &w = cx(i) > 0 ? xp : xn;
-                const int s = cx(i);
-                acc = fma(w.m1, f[r0 + x[2 + s]], acc);
-                acc = fma(w.p1, f[r0 + x[2 - s]], acc);
-                acc = fma(w.p2, f[r0 + x[2 - 2 * s]], acc);
-            }
-            if (cy(i) != 0) {
-                const Taps<R> &w = cy(i) > 0 ? yp : yn;
-                const int s = cy(i);
-                acc = fma(w.m1, f[y[2 + s] + x[2]], acc);
-                acc = fma(w.p1, f[y[2 - s] + x[2]], acc);
-                acc = fma(w.p2, f[y[2 - 2 * s] + x[2]], acc);
-            }
-            return acc;
-        } else {
-            // FP32: the difference first, so that the sum rounds to acc's size once
-            R d = R(0);
-            if (cx(i) != 0) {
-                const Taps<R> &w = cx(i) > 0 ? xp : xn;
-                const int s = cx(i);
-                d = w.c * v0;
-                d = fma(w.m1, f[r0 + x[2 + s]], d);
-                d = fma(w.p1, f[r0 + x[2 - s]], d);
-                d = fma(w.p2, f[r0 + x[2 - 2 * s]], d);
-            }
-            if (cy(i) != 0) {
-                const Taps<R> &w = cy(i) > 0 ? yp : yn;
-                const int s = cy(i);
-                d = cx(i) != 0 ? fma(w.c, v0, d) : w.c * v0;
-                d = fma(w.m1, f[y[2 + s] + x[2]], d);
-                d = fma(w.p1, f[y[2 - s] + x[2]], d);
-                d = fma(w.p2, f[y[2 - 2 * s] + x[2]], d);
-            }
-            return acc + d;
+        // one multiply-add per tap, the centre weights of a diagonal merged
+        if (cx(i) != 0 && cy(i) != 0) acc = fma((cx(i) > 0 ? xp.c : xn.c) + (cy(i) > 0 ? yp.c : yn.c), v0, acc);
+        else if (cx(i) != 0) acc = fma(cx(i) > 0 ? xp.c : xn.c, v0, acc);
+        else acc = fma(cy(i) > 0 ? yp.c : yn.c, v0, acc);
+        if (cx(i) != 0) {
+            const Taps<R> &w = cx(i) > 0 ? xp : xn;
+            const int s = cx(i);
+            acc = fma(w.m1, f[r0 + x[2 + s]], acc);
+            acc = fma(w.p1, f[r0 + x[2 - s]], acc);
+            acc = fma(w.p2, f[r0 + x[2 - 2 * s]], acc);
         }
+        if (cy(i) != 0) {
+            const Taps<R> &w = cy(i) > 0 ? yp : yn;
+            const int s = cy(i);
+            acc = fma(w.m1, f[y[2 + s] + x[2]], acc);
+            acc = fma(w.p1, f[y[2 - s] + x[2]], acc);
+            acc = fma(w.p2, f[y[2 - 2 * s] + x[2]], acc);
+        }
+        return acc;
     }
 };
 
@@ -556,7 +516,7 @@ __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
 }
 
 template <class R, bool FORCE>
-__global__ void __launch_bounds__(kThreads<R>) k_split_prepare(const SplitArgs<R> a)
+__global__ void __launch_bounds__(kThreads) k_split_prepare(const SplitArgs<R> a)
 {
     int x, y;
     if (!my_node<R, false>(a, x, y)) return;
@@ -574,12 +534,11 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_prepare(const SplitArgs<R
     }
 }
 
-// QUAD: four threads per node for every node; else for the wall nodes of an FP64
-// grid.
+// QUAD: four threads per node for every node; else for the wall nodes.
 template <class R, bool FORCE, bool WALLS, bool QUAD>
-__global__ void __launch_bounds__(kThreads<R>) k_split_star(const SplitArgs<R> a)
+__global__ void __launch_bounds__(kThreads) k_split_star(const SplitArgs<R> a)
 {
-    if (QUAD || (WALLS && kQuadWalls<R> && blockIdx.x < a.wall_blocks)) {
+    if (QUAD || (WALLS && blockIdx.x < a.wall_blocks)) {
         star_quad<R, FORCE, WALLS>(a);
         return;
     }
@@ -614,9 +573,9 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_star(const SplitArgs<R> a
 }
 
 template <class R, bool FORCE, bool WALLS, bool QUAD, bool LAST>
-__global__ void __launch_bounds__(kThreads<R>) k_split_update(const SplitArgs<R> a)
+__global__ void __launch_bounds__(kThreads) k_split_update(const SplitArgs<R> a)
 {
-    if (QUAD || (WALLS && kQuadWalls<R> && blockIdx.x < a.wall_blocks)) {
+    if (QUAD || (WALLS && blockIdx.x < a.wall_blocks)) {
         update_quad<R, FORCE, WALLS, LAST>(a);
         return;
     }
@@ -666,8 +625,8 @@ __global__ void __launch_bounds__(kThreads<R>) k_split_update(const SplitArgs<R>
 template <class R, class K>
 cudaError_t launch(K kernel, SplitArgs<R> a, int lanes, bool split_walls, bool chained, cudaStream_t s)
 {
-    constexpr int nt = kThreads<R>;
-    const int nodes = nt / lanes, wall_nodes = kQuadWalls<R> ? nt / 4 : nodes;  // per block
+    constexpr int nt = kThreads;
+    const int nodes = nt / lanes, wall_nodes = nt / 4;  // per block
     const int wx = split_walls && a.wx, wy = split_walls && a.wy;
     a.x0 = wx;
     a.y0 = wy;
@@ -710,22 +669,10 @@ cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStr
 
 // Weights of the mixed difference at one node of an axis, times `scale`, for
 // velocity sign +1 or -1: {k + s, k, k - s, k - 2s}; `central`: next to a wall.
-// In FP32 the taps go on the grid of weight_grid (lattice.cuh), on which the
-// centre, minus their sum, is exact: the update of a constant is exactly zero.
-template <class R>
-void taps(const Stencil<R> &st, bool central, double scale, R out[4])
+void taps(const Stencil<double> &st, bool central, double scale, double out[4])
 {
-    double t[3] = {double(st.wm1) * scale, double(st.w1) * scale, double(st.w2) * scale};
-    if (central) {
-        t[0] = 0.5 * scale;
-        t[1] = -0.5 * scale;
-        t[2] = 0.0;
-    }
-    if (sizeof(R) == 4 && scale != 0.0) {
-        const double q = std::ldexp(1.0, std::ilogb(scale) - 21);
-        for (double &v : t) v = std::nearbyint(v / q) * q;
-    }
-    const R m1 = R(t[0]), p1 = R(t[1]), p2 = R(t[2]);
+    const double m1 = scale * (central ? 0.5 : st.wm1), p1 = scale * (central ? -0.5 : st.w1);
+    const double p2 = scale * (central ? 0.0 : st.w2);
     out[0] = m1;
     out[1] = -((m1 + p1) + p2);
     out[2] = p1;
@@ -734,15 +681,14 @@ void taps(const Stencil<R> &st, bool central, double scale, R out[4])
 
 }  // namespace
 
-size_t split_table_bytes(int nx, int ny, size_t real_size) { return 16 * (size_t)(nx + ny) * real_size; }
+size_t split_table_bytes(int nx, int ny) { return 16 * (size_t)(nx + ny) * sizeof(double); }
 
 // The tables in the order bx, by, cx, cy: [n][2][4] each.
-template <class R>
-std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
-                                 double beta, double h, double dt)
+std::vector<double> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
+                                      double beta, double h, double dt)
 {
-    const Stencil<R> st = make_stencil<R>(beta);
-    std::vector<R> out;
+    const Stencil<double> st = make_stencil<double>(beta);
+    std::vector<double> out;
     out.reserve(16 * (mx.size() + my.size()));
     auto axis = [&](const std::vector<double> &m, bool wall, double s) {
         const int n = (int)m.size();
@@ -750,8 +696,8 @@ std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vecto
             for (int sign = 1; sign >= -1; sign -= 2) {
                 // the second-order upwind tap k - 2 s would leave the domain
                 const bool central = wall && (sign > 0 ? k < 2 : k > n - 3);
-                R t[4];
-                taps<R>(st, central, -s * double(R(m[k])), t);
+                double t[4];
+                taps(st, central, -s * m[k], t);
                 out.insert(out.end(), t, t + 4);
             }
     };
@@ -761,20 +707,18 @@ std::vector<R> make_split_tables(const std::vector<double> &mx, const std::vecto
     axis(my, wy, dt);
     return out;
 }
-template std::vector<float> make_split_tables<float>(const std::vector<double> &, const std::vector<double> &, bool,
-                                                     bool, double, double, double);
-template std::vector<double> make_split_tables<double>(const std::vector<double> &, const std::vector<double> &, bool,
-                                                       bool, double, double, double);
 
-// nsteps steps of the state in s.gin, in place.
 // Grids of at most so many nodes take four threads per node throughout: up to two
 // such warps per scheduler of 152 SMs on a periodic grid, one on a walled one
 // (us per step, four threads against one: 24^2 6.4 / 11.7, 64^2 7.1 / 11.6, 96^2
 // 10.9 / 12.5, 120^2 15.1 / 13.0; walled 65^2 10.6 / 13.2, 97^2 14.2 / 13.6).
 constexpr long long kQuadNodes = 9728, kQuadWalledNodes = 4864;
-template <class R>
-cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, int nsteps, cudaStream_t stream)
+
+// nsteps steps of the state in s.gin, in place.
+cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, int nsteps,
+                         cudaStream_t stream)
 {
+    using R = double;
     if (nsteps <= 0) return cudaSuccess;
     SplitArgs<R> a{};
     a.P = const_cast<R *>(s.gin);
@@ -806,13 +750,8 @@ cudaError_t launch_split(const StepArgs<R> &s, R *Q0, R *Q1, const R *tables, in
         if (walls) return s.force ? go(y, y, quad) : go(n, y, quad);
         return s.force ? go(y, n, quad) : go(n, n, quad);
     };
-    if constexpr (sizeof(R) == 8) {
-        if ((long long)a.nx * a.ny <= (walls ? kQuadWalledNodes : kQuadNodes)) return pick(std::true_type{});
-    }
+    if ((long long)a.nx * a.ny <= (walls ? kQuadWalledNodes : kQuadNodes)) return pick(std::true_type{});
     return pick(std::false_type{});
 }
-template cudaError_t launch_split<float>(const StepArgs<float> &, float *, float *, const float *, int, cudaStream_t);
-template cudaError_t launch_split<double>(const StepArgs<double> &, double *, double *, const double *, int,
-                                          cudaStream_t);
 
 }  // namespace fdlbm

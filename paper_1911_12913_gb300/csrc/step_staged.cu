@@ -1,11 +1,11 @@
-// Staged T2S2-FDLBM2 step of single grids, for any boundary combination: the
+// Staged T2S2-FDLBM step of single grids, for any boundary combination: the
 // stages of Sec. 2D run as separate kernels through three scratch fields P, Q,
 // S, one thread per node (stage bodies in staged_nodes.cuh).  This path serves
-// walled grids in FP64 and grids too small for the fused kernels' halo
-// (T2S2-FDLBM1 takes step_split.cu there).
+// T2S2-FDLBM2 on walled grids in FP64, FP32 grids too small for the fused
+// kernels' halo, and path = STAGED (in FP64, T2S2-FDLBM1 takes step_split.cu).
 //
-// Launch order per step: prepare (all nodes), [with walls: Eq. 3.10 on P], star
-// (interior), Eq. 3.10 on S, update (interior), Eq. 3.10 on the
+// Launch order per step: prepare (all nodes), [scheme 2 with walls: Eq. 3.10
+// on P], star (interior), Eq. 3.10 on S, update (interior), Eq. 3.10 on the
 // new state.
 #include "staged_nodes.cuh"
 
@@ -50,7 +50,7 @@ cudaError_t run(const StepArgs<R> &a, cudaStream_t s)
     const int nwall = wall_count(a);
     const bool walls = nwall > 0;
     k_prepare<R, FORCE><<<grd, blk, 0, s>>>(a);
-    if (walls)
+    if (walls && a.scheme == FDLBM_SCHEME_T2S2_2)
         k_wall_nee<R, false><<<(nwall + 127) / 128, 128, 0, s>>>(a, a.P, R(0));
     k_star<R, FORCE><<<grd, blk, 0, s>>>(a);
     if (walls) k_wall_nee<R, false><<<(nwall + 127) / 128, 128, 0, s>>>(a, a.S, R(0));

@@ -14,10 +14,9 @@
 // Walls: wall nodes belong to the tile of their interior neighbour x_j.  In
 // tiles that touch a wall, Eq. 3.10 runs for all their wall nodes together
 // after stage B (f*) and after stage C (the new f~), one thread per wall node,
-// and the difference is written as a central part and an upwind correction,
-// whose weight is zero next to a wall where it would leave the domain.  Outside
-// a walled domain, loads read the nearest node; zero weights meet those values,
-// which are finite.
+// and columns and rows next to a wall, where the upwind difference would leave
+// the domain, select the central one.  Outside a walled domain, loads read the
+// nearest node; no stored value depends on those.
 //
 // What bounds it: at 1024^2 (27 us per step, 39 GLUPS) the shared-memory pipe,
 // about 65 % busy with 38 64-bit loads per pair and stage; issue slots 43 % busy.
@@ -46,11 +45,12 @@ struct TileSmem {
     float mx[2 * kAP], my[kAR];  // metrics of stage A's region
 };
 
-// Weights of the mixed difference in one axis times -s m, for the columns of
-// the pair (or one row, twice).  The plain form holds the scale; the edge form
-// the central and the upwind weight, the latter for both signs.
+// Scale -s m of the difference in one axis for the columns of the pair (or one
+// row, twice), and the columns where the difference of a sign is the central one
+// alone (edge tiles).
 struct Diff {
-    f2 k1, k2p, k2n;
+    f2 k;
+    bool p0, p1, n0, n1;
 };
 
 // An output rectangle [x0, x1) x [y0, y1) that another launch writes.
@@ -154,29 +154,33 @@ struct Tile {
     {
         const f2 mx = *reinterpret_cast<const f2 *>(&sm.mx[x - x0 + 4]);
         const float my = sm.my[y - y0 + 4];
-        dx.k1 = mul2(bc(-s), mx);
-        dy.k1 = bc(-s * my);
-        if (EDGE) {  // central: k1/2; upwind correction: k1 beta/2, none next to a wall
-            const f2 ux = mul2(dx.k1, w[3]), uy = mul2(dy.k1, w[3]);
-            dx.k2p = make_float2(wx && x <= 1 ? 0.f : ux.x, wx && x + 1 <= 1 ? 0.f : ux.y);
-            dx.k2n = make_float2(wx && x >= a.nx - 2 ? 0.f : ux.x, wx && x + 1 >= a.nx - 2 ? 0.f : ux.y);
-            dy.k2p = wy && y <= 1 ? bc(0.f) : uy;
-            dy.k2n = wy && y >= a.ny - 2 ? bc(0.f) : uy;
-            dx.k1 = mul2(dx.k1, bc(0.5f));
-            dy.k1 = mul2(dy.k1, bc(0.5f));
+        dx.k = mul2(bc(-s), mx);
+        dy.k = bc(-s * my);
+        if (EDGE) {
+            dx.p0 = wx && x <= 1;
+            dx.p1 = wx && x + 1 <= 1;
+            dx.n0 = wx && x >= a.nx - 2;
+            dx.n1 = wx && x + 1 >= a.nx - 2;
+            dy.p0 = dy.p1 = wy && y <= 1;
+            dy.n0 = dy.n1 = wy && y >= a.ny - 2;
         }
     }
 
     // acc - s xi_a d/dx_a of one axis, from the taps at 0, +1, -1, -2 along the
-    // velocity: the difference first, so that the sum rounds to acc's size once
+    // velocity: the difference first, so that the sum rounds to acc's size once.
+    // Edge tiles take the same weights as the others: their rounding (2^-22)
+    // scales the advection speed by up to 5e-7, and a tile with other roundings
+    // would be a source at its rim (257^2 cavity, 30,000 steps: 1.4e-5 off FP64
+    // with a central part and an upwind correction of its own weight).
     template <bool EDGE>
-    __device__ __forceinline__ f2 axis(f2 v0, f2 up, f2 dn, f2 dn2, f2 k1, f2 k2, f2 acc) const
+    __device__ __forceinline__ f2 axis(f2 v0, f2 up, f2 dn, f2 dn2, f2 k, bool c0, bool c1, f2 acc) const
     {
+        f2 d = fma2(w[3], dn2, fma2(w[2], dn, fma2(w[0], up, mul2(w[1], v0))));
         if (EDGE) {
-            acc = fma2(k1, sub2(up, dn), acc);
-            return fma2(k2, fma2(bc(3.f), sub2(v0, dn), sub2(dn2, up)), acc);
+            const f2 c = mul2(bc(0.5f), sub2(up, dn));
+            d = make_float2(c0 ? c.x : d.x, c1 ? c.y : d.y);
         }
-        return fma2(k1, fma2(w[3], dn2, fma2(w[2], dn, fma2(w[0], up, mul2(w[1], v0)))), acc);
+        return fma2(k, d, acc);
     }
 
     // acc - s xi.grad of population i from its plane f at o (row stride W).
@@ -186,11 +190,11 @@ struct Tile {
         if (cx(i) != 0) {
             const f2 L = f[o - 1], R = f[o + 1];
             const f2 lo = make_float2(L.y, v0.x), hi = make_float2(v0.y, R.x);
-            if (cx(i) > 0) acc = axis<EDGE>(v0, hi, lo, L, dx.k1, dx.k2p, acc);
-            else acc = axis<EDGE>(v0, lo, hi, R, dx.k1, dx.k2n, acc);
+            if (cx(i) > 0) acc = axis<EDGE>(v0, hi, lo, L, dx.k, dx.p0, dx.p1, acc);
+            else acc = axis<EDGE>(v0, lo, hi, R, dx.k, dx.n0, dx.n1, acc);
         }
-        if (cy(i) > 0) acc = axis<EDGE>(v0, f[o + W], f[o - W], f[o - 2 * W], dy.k1, dy.k2p, acc);
-        if (cy(i) < 0) acc = axis<EDGE>(v0, f[o - W], f[o + W], f[o + 2 * W], dy.k1, dy.k2n, acc);
+        if (cy(i) > 0) acc = axis<EDGE>(v0, f[o + W], f[o - W], f[o - 2 * W], dy.k, dy.p0, dy.p1, acc);
+        if (cy(i) < 0) acc = axis<EDGE>(v0, f[o - W], f[o + W], f[o + 2 * W], dy.k, dy.n0, dy.n1, acc);
         return acc;
     }
 

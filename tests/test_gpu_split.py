@@ -1,5 +1,5 @@
-"""The step in two launches (step_split.cu), which FP64 grids take by default
-and path="staged" in both precisions, against the oracle (four threads per node on
+"""The FP64 step in two launches (step_split.cu), the automatic choice and
+path="staged", against the oracle (four threads per node on
 small FP64 grids and at FP64 wall nodes): strips of one column
 to several, partial last warps and strips, grids of three nodes per axis, every
 boundary combination with moving walls, random metrics, a force field, the
@@ -21,9 +21,9 @@ if not torch.cuda.is_available():
 
 from paper_1911_12913_gb300.solver import FDLBM  # noqa: E402
 
-# The bounds of the other step kernels: 12 steps of O(1e-16) (FP64) and
-# O(2^-24 of the deviations) (FP32) roundings, with the margin used there.
-BOUNDS = {"fp64": (1e-12, 1e-11), "fp32": (1e-7, 2e-5)}
+# The bounds of the other FP64 step kernels: 12 steps of O(1e-16) roundings, with
+# the margin used there.
+L2, DEV = 1e-12, 1e-11
 
 
 def _axis(kind, n, seed, length):
@@ -34,7 +34,7 @@ def _axis(kind, n, seed, length):
     return I.tanh_axis(n - 1, 1.5) if length == 1.0 else I.wall_axis(n - 1, 0.0, length)
 
 
-@pytest.mark.parametrize("precision", ["fp64", "fp32"])
+@pytest.mark.parametrize("path", ["auto", "staged"])
 @pytest.mark.parametrize("x,y,nx,ny,more", [
     ("periodic", "periodic", 3, 3, {}), ("wall", "wall", 3, 3, {}), ("wall", "periodic", 3, 7, {}),
     ("periodic", "wall", 4, 3, {}), ("periodic", "periodic", 31, 33, {"force": True}),
@@ -50,16 +50,15 @@ def _axis(kind, n, seed, length):
     ("periodic", "periodic", 128, 76, {}), ("periodic", "periodic", 139, 70, {}), ("wall", "wall", 76, 64, {}),
     ("wall", "wall", 65, 75, {}),
 ])
-def test_split_step_matches_oracle(precision, x, y, nx, ny, more):
+def test_split_step_matches_oracle(path, x, y, nx, ny, more):
     xa, ya = _axis(x, nx, 31, 1.0), _axis(y, ny, 32, 0.8)
     rng = np.random.default_rng(nx * 1000 + ny)
     force = 1e-3 * rng.uniform(-1, 1, size=(2, ny, nx)) if more.get("force") else None
     wall_u = [tuple(0.05 * rng.uniform(-1, 1, size=2)) for _ in range(4)]
     eq, A = more.get("eq", "standard"), more.get("A", 0.5)
-    s = FDLBM(xa, ya, nu=0.02, cfl=0.3, blend=0.2, A=A, precision=precision, has_force=force is not None,
-              wall_u=wall_u, equilibrium=eq, path="auto" if precision == "fp64" else "staged",
-              graph_steps=more.get("graph", 0))
-    assert s.describe.startswith("split " + precision), s.describe
+    s = FDLBM(xa, ya, nu=0.02, cfl=0.3, blend=0.2, A=A, has_force=force is not None,
+              wall_u=wall_u, equilibrium=eq, path=path, graph_steps=more.get("graph", 0))
+    assert s.describe.startswith("split fp64"), s.describe
     assert s.kernels_per_step == 2
     o = O.Oracle(xa, ya, nu=0.02, dt=s.dt, beta=0.2, A=A, force=force, wall_u=wall_u,
                  incomp=eq == "incompressible")
@@ -74,8 +73,7 @@ def test_split_step_matches_oracle(precision, x, y, nx, ny, more):
         o.step(n)
     s.sync()
     assert s.steps_done == 12
-    l2, dev = BOUNDS[precision]
-    assert_parity(s.get_state(), o.f, l2=l2, dev=dev, label=f"{s.describe} {x}/{y} {nx}x{ny}")
+    assert_parity(s.get_state(), o.f, l2=L2, dev=DEV, label=f"{s.describe} {x}/{y} {nx}x{ny}")
 
 
 def test_split_step_is_the_automatic_choice_for_fp64_only():
@@ -90,3 +88,4 @@ def test_split_step_is_the_automatic_choice_for_fp64_only():
     assert FDLBM(pa, pa, path="fused", **kw).describe.startswith("fused fp64")
     assert FDLBM(pa, pa, scheme=2, **kw).describe.startswith("fused-scheme2")
     assert not FDLBM(pa, pa, precision="fp32", **kw).describe.startswith("split")
+    assert FDLBM(wa, wa, precision="fp32", path="staged", **kw).describe.startswith("staged fp32dev")
