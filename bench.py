@@ -39,12 +39,10 @@ N_GRID = 4096
 # unstable at the 4096^2 spacing (dt/tau = 0.026, nearly collisionless transport).
 NU, CFL, BLEND, U0, SEED = 0.001, 0.5, 0.1, 0.01, 2026
 BYTES_PER_CELL = {"fp32": 72, "fp64": 144}   # 9 populations read once + written once
-# FP64 is bound by the FP64 units, not HBM.  The FP64 fused step executes
-# 80.0 M DADD + 60.3 M DMUL + 212.5 M DFMA thread instructions per 1,474,560
-# thread-rows (ncu, 1024^2, 9 x 32 CTAs of 128 threads x 40 rows): 383 flop
-# per node of sweep work, the algorithmic figure per cell update (the halo
-# recompute of a given tiling comes on top).
-FP64_FLOP_PER_CELL = 383
+# FP64 is bound by the FP64 units, not HBM.  The split step executes 58 DADD + 28
+# DMUL + 141 DFMA thread instructions per node and step (ncu, 1024^2, star plus
+# update kernel): 368 flop, each quantity formed once.
+FP64_FLOP_PER_CELL = 368
 FP64_NOMINAL_TFLOPS = 1.25   # GB300 nominal FP64 rate (non-tensor), context only
 SAMPLE_N = 512                                # oracle sample grid
 
