@@ -170,8 +170,9 @@ struct Tile {
     // velocity: the difference first, so that the sum rounds to acc's size once.
     // Edge tiles take the same weights as the others: their rounding (2^-22)
     // scales the advection speed by up to 5e-7, and a tile with other roundings
-    // would be a source at its rim (257^2 cavity, 30,000 steps: 1.4e-5 off FP64
-    // with a central part and an upwind correction of its own weight).
+    // would be a source at its rim.  The gain is small: 257^2 cavity, 30,000 steps
+    // from its steady state, 1.33e-5 off FP64 against 1.4e-5 with a central part
+    // and an upwind correction of its own weight (walls sweep 5.7e-6).
     template <bool EDGE>
     __device__ __forceinline__ f2 axis(f2 v0, f2 up, f2 dn, f2 dn2, f2 k, bool c0, bool c1, f2 acc) const
     {
