@@ -499,7 +499,9 @@ template <bool FORCE, bool UNI>
 __global__ void __launch_bounds__(kNT, 2) k_adj_tile(const __grid_constant__ AdjTileArgs q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    AdjTile<FORCE, UNI>(q, *reinterpret_cast<AdjSmem *>(smem_raw), blockIdx.x, blockIdx.y).run();
+    // linear over the tiles: a grid may have more rows of tiles than gridDim.y allows
+    const int tx = tiles_along(q.a.nx, false, kTX), by = blockIdx.x / tx;
+    AdjTile<FORCE, UNI>(q, *reinterpret_cast<AdjSmem *>(smem_raw), blockIdx.x - by * tx, by).run();
     chain_next();
 }
 
@@ -521,7 +523,8 @@ cudaError_t launch_adjoint_tile(const StepArgs<float> &a, bool uniform, const fl
                         : (uniform ? k_adj_tile<false, true> : k_adj_tile<false, false>);
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjSmem));
     if (e != cudaSuccess) return e;
-    return chained_launch(kern, dim3((a.nx + kTX - 1) / kTX, (a.ny + kTY - 1) / kTY), kNT, sizeof(AdjSmem), s, q);
+    return chained_launch(kern, dim3(tiles_along(a.nx, false, kTX) * tiles_along(a.ny, false, kTY)), kNT,
+                          sizeof(AdjSmem), s, q);
 }
 
 }  // namespace fdlbm

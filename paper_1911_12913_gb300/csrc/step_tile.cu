@@ -442,7 +442,9 @@ template <bool FORCE, bool WALLS>
 __global__ void __launch_bounds__(kNT, kMinBlocks) k_step_tile(const __grid_constant__ StepArgs<float> a)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    tile_step<FORCE, WALLS>(a, smem_raw, blockIdx.x, blockIdx.y);
+    // linear over the tiles: a grid may have more rows of tiles than gridDim.y allows
+    const int tx = tiles_along(a.nx, a.bc_x == FDLBM_WALL, kTX), by = blockIdx.x / tx;
+    tile_step<FORCE, WALLS>(a, smem_raw, blockIdx.x - by * tx, by);
 }
 
 // The frame of a walled grid: the tiles that hold nodes outside `skip`, the
@@ -506,11 +508,10 @@ __global__ void __launch_bounds__(kNT, kMinBlocks)
 
 }  // namespace
 
-// Tiles of a grid; wall nodes go with their interior neighbour's tile.
 void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty)
 {
-    *tx = (nx - (wall_x ? 1 : 0) + kTX - 1) / kTX;
-    *ty = (ny - (wall_y ? 1 : 0) + kTY - 1) / kTY;
+    *tx = tiles_along(nx, wall_x, kTX);
+    *ty = tiles_along(ny, wall_y, kTY);
 }
 
 cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s)
@@ -523,7 +524,7 @@ cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s)
     if (e != cudaSuccess) return e;
     int tx, ty;
     tile_counts(a.nx, a.ny, a.bc_x == FDLBM_WALL, a.bc_y == FDLBM_WALL, &tx, &ty);
-    return chained_launch(kern, dim3(tx, ty), kNT, smem, s, a);
+    return chained_launch(kern, dim3(tx * ty), kNT, smem, s, a);
 }
 
 // The nodes of a walled grid outside the rectangle [x0, x1) x [y0, y1).

@@ -16,6 +16,13 @@ constexpr int kBP = kTP + 2, kBR = kTY + 4;       // region of stage B
 constexpr int kARing = kAP * kAR - kNT, kBRing = kBP * kBR - kNT;  // pairs around the tile
 static_assert(kARing <= kNT && kBRing <= kNT, "one pass over the ring");
 
+// Tiles of `size` nodes along an axis of n; a wall node goes with its interior
+// neighbour's tile.
+__host__ __device__ __forceinline__ int tiles_along(int n, bool wall, int size)
+{
+    return (n - (wall ? 1 : 0) + size - 1) / size;
+}
+
 // Index k of an axis of n nodes: wrapped on a periodic axis, the nearest node
 // on a walled one.
 __device__ __forceinline__ int axis_index(int k, int n, bool wall)
