@@ -84,8 +84,10 @@ enum { FDLBM_EQ_STANDARD = 0, FDLBM_EQ_INCOMPRESSIBLE = 1 };
  * field, any size where WARP does not apply).  Beyond that it picks WARP where
  * it applies, on a walled grid with the frame on the tile kernel (T2S2-FDLBM1),
  * and SCALAR otherwise; with path FUSED or a tile height given, WARP
- * where it applies, except on walled grids of fewer than 1.5 M nodes, where the
- * frame launch's fixed cost makes the walls sweep faster, and SCALAR otherwise.
+ * where it applies, except on walled grids of fewer than 1.5 x 2^20 nodes, where
+ * the frame launch's fixed cost makes the walls sweep faster, and SCALAR
+ * otherwise.  T2S2-FDLBM2 takes WARP where it applies, except on walled grids of
+ * fewer than 1.25 M nodes (1.5 x 2^20 where a side has fewer than 256 nodes).
  * Asking for a variant that does not apply returns FDLBM_EUNSUPPORTED; the
  * values 2 to 4 are not used. */
 enum { FDLBM_VARIANT_AUTO = 0, FDLBM_VARIANT_SCALAR = 1, FDLBM_VARIANT_WARP = 5 };

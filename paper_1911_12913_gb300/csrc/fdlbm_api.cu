@@ -115,6 +115,19 @@ double tile_walled_nodes(const fdlbm_opts *o, bool batch)
     return o->has_force ? 1.7e6 : 1.25e6;
 }
 
+// Walled T2S2-FDLBM2 grids (FP32) of fewer nodes run on the walls sweep rather
+// than on the warp tile with its frame, with and without a force field.  us per
+// step on GB300, sweep against warp tile:
+//   walls in x and y  1120^2 91.4 / 62.9, forced 108.2 / 94.3; 4500 x 300 85.6 / 65.6
+//   in x              1152^2 97.4 / 72.6, forced 121.9 / 98.8
+//   in y              1152^2 66.7 / 65.5, forced 89.1 / 89.1; 768^2 35.2 / 40.0
+// A thin grid is mostly frame (66 x 20000 126 / 210, 20000 x 66 76 / 167): its
+// line lies at 1.5 x 2^20 nodes.
+double warp_walled_nodes_s2(const fdlbm_grid *g)
+{
+    return std::min(g->nx, g->ny) < 256 ? 1.5 * 1048576 : 1.25e6;
+}
+
 // T2S2-FDLBM1 in FP32 on the tile kernel (step_tile.cu) unless a tile height or
 // a kernel is asked for: a step of it lasts 4-5 us on the smallest grids, where
 // the sweeps walk a chain of ten dependent rows, and runs at 36-38 GLUPS (31
@@ -537,7 +550,9 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     // height is asked for, below about 1.5 M nodes on the walls sweep
     // (2049^2 cavity 164 us per step against 95 on the warp tile)
     const bool auto_all = o.path == FDLBM_PATH_AUTO && o.rows_per_cta == 0;
-    const double small_nodes = force_staged || auto_all ? tile_walled_nodes(&o, force_staged) : 1.5 * 1048576;
+    const double small_nodes = !s1                        ? warp_walled_nodes_s2(g)
+                               : force_staged || auto_all ? tile_walled_nodes(&o, force_staged)
+                                                          : 1.5 * 1048576;
     const bool small_walled = walled(g) && (double)g->nx * g->ny < small_nodes;
     if (variant == FDLBM_VARIANT_AUTO)
         variant = warp_ok && !small_walled ? FDLBM_VARIANT_WARP : FDLBM_VARIANT_SCALAR;
