@@ -22,6 +22,7 @@
 // thread and tile).  Against the sweep of adjoint.cu, which walks a chain of
 // rows in scalar arithmetic, us per step on GB300, with a force field: 256^2
 // 18.4 -> 7.4, 512^2 19.6, 2048^2 360 -> 254, 4096^2 1288 -> 1007.
+#include <algorithm>
 #include <cstdint>
 
 #include "internal.h"
@@ -46,6 +47,7 @@ struct AdjTileArgs {
     const float *lam_next;
     float *lam_prev;
     double *dforce;
+    int row0;  // first row of tiles of the launch (TALL)
 };
 
 // Lattice moments sum w_i (1, 3x, 3y, xx, xy, yy, xxy, xyy) v_i of a cotangent.
@@ -495,13 +497,13 @@ struct AdjTile {
     }
 };
 
-template <bool FORCE, bool UNI>
+// TALL: a launch for the rows of tiles from row0 on.
+template <bool FORCE, bool UNI, bool TALL>
 __global__ void __launch_bounds__(kNT, 2) k_adj_tile(const __grid_constant__ AdjTileArgs q)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // linear over the tiles: a grid may have more rows of tiles than gridDim.y allows
-    const int tx = tiles_along(q.a.nx, false, kTX), by = blockIdx.x / tx;
-    AdjTile<FORCE, UNI>(q, *reinterpret_cast<AdjSmem *>(smem_raw), blockIdx.x - by * tx, by).run();
+    const int by = blockIdx.y + (TALL ? q.row0 : 0);
+    AdjTile<FORCE, UNI>(q, *reinterpret_cast<AdjSmem *>(smem_raw), blockIdx.x, by).run();
     chain_next();
 }
 
@@ -518,13 +520,16 @@ bool adjoint_tile_ok(const void *state, const void *lam_next, const void *lam_pr
 cudaError_t launch_adjoint_tile(const StepArgs<float> &a, bool uniform, const float *lam_next, float *lam_prev,
                                 double *dforce, cudaStream_t s)
 {
-    const AdjTileArgs q{a, lam_next, lam_prev, dforce};
-    auto kern = a.force ? (uniform ? k_adj_tile<true, true> : k_adj_tile<true, false>)
-                        : (uniform ? k_adj_tile<false, true> : k_adj_tile<false, false>);
+    AdjTileArgs q{a, lam_next, lam_prev, dforce, 0};
+    const int tx = tiles_along(a.nx, false, kTX), ty = tiles_along(a.ny, false, kTY);
+    auto kern = a.force ? (uniform ? k_adj_tile<true, true, false> : k_adj_tile<true, false, false>)
+                        : (uniform ? k_adj_tile<false, true, false> : k_adj_tile<false, false, false>);
+    if (ty > kMaxTileRows) kern = a.force ? k_adj_tile<true, false, true> : k_adj_tile<false, false, true>;
     cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)sizeof(AdjSmem));
     if (e != cudaSuccess) return e;
-    return chained_launch(kern, dim3(tiles_along(a.nx, false, kTX) * tiles_along(a.ny, false, kTY)), kNT,
-                          sizeof(AdjSmem), s, q);
+    for (; q.row0 < ty && e == cudaSuccess; q.row0 += kMaxTileRows)
+        e = chained_launch(kern, dim3(tx, std::min(ty - q.row0, kMaxTileRows)), kNT, sizeof(AdjSmem), s, q);
+    return e;
 }
 
 }  // namespace fdlbm

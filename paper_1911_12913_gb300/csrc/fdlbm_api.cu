@@ -928,7 +928,7 @@ int fdlbm_kernels_per_step(fdlbm_t h)
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
     if (h->split) return 2;  // and one more per fdlbm_step call (or graph replay)
     if (h->path == FDLBM_PATH_FUSED) {
-        if (h->tile) return 1;
+        if (h->tile) return tile_launches(h->nx, h->ny, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL);
         // a walled grid on the warp-tile kernel: the frame's launch and the interior's
         if (h->precision == FDLBM_FP32_DEV && h->variant == FDLBM_VARIANT_WARP && walls) {
             int interior = 0, frame = 0;

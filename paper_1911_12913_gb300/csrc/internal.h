@@ -189,6 +189,7 @@ cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, cons
                          cudaStream_t stream);
 // step_tile.cu (FP32 T2S2-FDLBM1, one launch per step, a tile per block)
 void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty);
+int tile_launches(int nx, int ny, bool wall_x, bool wall_y);  // of one step
 cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s);
 cudaError_t launch_frame_tile(const StepArgs<float> &a, int x0, int x1, int y0, int y1, cudaStream_t s);
 cudaError_t launch_batched_tile(const BatchTables &t, int parity, int blk_off, int nblocks, cudaStream_t s);

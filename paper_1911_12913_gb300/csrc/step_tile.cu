@@ -438,13 +438,13 @@ __device__ __forceinline__ void tile_step(const StepArgs<float> &a, unsigned cha
     chain_next();
 }
 
-template <bool FORCE, bool WALLS>
-__global__ void __launch_bounds__(kNT, kMinBlocks) k_step_tile(const __grid_constant__ StepArgs<float> a)
+// TALL: a launch for the rows of tiles from row0 on.
+template <bool FORCE, bool WALLS, bool TALL>
+__global__ void __launch_bounds__(kNT, kMinBlocks)
+    k_step_tile(const __grid_constant__ StepArgs<float> a, const int row0)
 {
     extern __shared__ __align__(16) unsigned char smem_raw[];
-    // linear over the tiles: a grid may have more rows of tiles than gridDim.y allows
-    const int tx = tiles_along(a.nx, a.bc_x == FDLBM_WALL, kTX), by = blockIdx.x / tx;
-    tile_step<FORCE, WALLS>(a, smem_raw, blockIdx.x - by * tx, by);
+    tile_step<FORCE, WALLS>(a, smem_raw, blockIdx.x, blockIdx.y + (TALL ? row0 : 0));
 }
 
 // The frame of a walled grid: the tiles that hold nodes outside `skip`, the
@@ -514,17 +514,27 @@ void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty)
     *ty = tiles_along(ny, wall_y, kTY);
 }
 
+int tile_launches(int nx, int ny, bool wall_x, bool wall_y)
+{
+    int tx, ty;
+    tile_counts(nx, ny, wall_x, wall_y, &tx, &ty);
+    return (ty + kMaxTileRows - 1) / kMaxTileRows;
+}
+
 cudaError_t launch_tile(const StepArgs<float> &a, cudaStream_t s)
 {
     const bool walls = a.bc_x == FDLBM_WALL || a.bc_y == FDLBM_WALL;
     const size_t smem = a.force ? sizeof(TileSmem<true>) : sizeof(TileSmem<false>);
-    auto kern = a.force ? (walls ? k_step_tile<true, true> : k_step_tile<true, false>)
-                        : (walls ? k_step_tile<false, true> : k_step_tile<false, false>);
-    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
-    if (e != cudaSuccess) return e;
     int tx, ty;
     tile_counts(a.nx, a.ny, a.bc_x == FDLBM_WALL, a.bc_y == FDLBM_WALL, &tx, &ty);
-    return chained_launch(kern, dim3(tx * ty), kNT, smem, s, a);
+    auto kern = a.force ? (walls ? k_step_tile<true, true, false> : k_step_tile<true, false, false>)
+                        : (walls ? k_step_tile<false, true, false> : k_step_tile<false, false, false>);
+    if (ty > kMaxTileRows) kern = a.force ? k_step_tile<true, true, true> : k_step_tile<false, true, true>;
+    cudaError_t e = cudaFuncSetAttribute(kern, cudaFuncAttributeMaxDynamicSharedMemorySize, (int)smem);
+    if (e != cudaSuccess) return e;
+    for (int row0 = 0; row0 < ty && e == cudaSuccess; row0 += kMaxTileRows)
+        e = chained_launch(kern, dim3(tx, std::min(ty - row0, kMaxTileRows)), kNT, smem, s, a, row0);
+    return e;
 }
 
 // The nodes of a walled grid outside the rectangle [x0, x1) x [y0, y1).

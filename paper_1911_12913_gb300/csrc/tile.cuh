@@ -23,6 +23,13 @@ __host__ __device__ __forceinline__ int tiles_along(int n, bool wall, int size)
     return (n - (wall ? 1 : 0) + size - 1) / size;
 }
 
+// Rows of tiles of one launch (the limit of gridDim.y).  A taller grid takes more
+// launches of an instance of its own, each with its first row as an argument: in
+// the common instance that argument cost the adjoint 0.7 % (2048^2 rollout), and
+// one launch over a linear block index, with a division per block, made the forced
+// step spill (1000^2 34.1 us against 32.1).
+constexpr int kMaxTileRows = 65535;
+
 // Index k of an axis of n nodes: wrapped on a periodic axis, the nearest node
 // on a walled one.
 __device__ __forceinline__ int axis_index(int k, int n, bool wall)

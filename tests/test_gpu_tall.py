@@ -34,6 +34,7 @@ def test_tile_step_on_a_tall_walled_grid():
         out[variant] = s.get_state()
         kernel = s.describe.split()[0]
         assert kernel == ("fused-tile" if variant == "auto" else "fused-walls"), kernel
+        assert s.kernels_per_step == (2 if variant == "auto" else 1)
         s.close()
     assert_parity(out["auto"], out["scalar"], l2=L2, dev=DEV, label=f"{NX}x{NY}")
 
