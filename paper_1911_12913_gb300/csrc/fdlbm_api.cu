@@ -143,9 +143,22 @@ double warp_walled_nodes_s2(const fdlbm_grid *g)
 //                  1536 x 1537 78.9 / 68
 //   warp tile, frame as a walls sweep (a batch)
 //                  1025^2 29.2 / 44.5, 2049^2 115 / 95, forced 2048 x 2049 134 / 137
-// The lines below lie where the two cross.  On periodic grids the warp tile, where
-// it applies, also keeps the thin ones that fill less than 0.7 of their tiles
-// (300 x 33: the choice that fdlbm_describe has always shown for it).
+// Walled lines: where the two cross.  On a periodic grid the tile kernel's time
+// goes with the nodes of its whole tiles, the warp tile's with the grid's and a
+// larger fixed cost, the scalar sweep's with the nodes of its whole strips, so
+// the lines compare these (further us per step, tile kernel against the other;
+// near a line the kept one is at most 9 % behind):
+//   warp tile      68^2 3.8 / 9.0, 100^2 3.8 / 9.1, 4096 x 33 6.4 / 10.7, 580 x 1000 16.6 / 17.8,
+//                  644 x 1000 18.1 / 17.4, 772 x 1000 21.4 / 19.3, 196 x 3500 21.8 / 19.2,
+//                  100 x 7000 25.3 / 20.1
+//     forced       100^2 4.5 / 11.5, 100 x 4000 18.6 / 21.2, 772 x 1000 25.8 / 28.8,
+//                  100 x 7000 30.5 / 28.6, 20000 x 33 29.0 / 26.4
+//   scalar sweep   33 x 30000 52.5 / 66.3, 5001 x 200 26.9 / 25.7, 10001 x 33 13.6 / 12.7,
+//                  30001 x 33 35.9 / 26.6, forced 45.1 / 35.7
+// Thin grids that fill less than 0.65 of their tiles stay on the warp tile, the
+// automatic choice that tests hold for one of them, although the tile kernel
+// measures faster there too while the tiles are few (300 x 33 3.7 / 8.9, 8192 x 17
+// 8.3 / 10.6).
 bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
 {
     if (o->scheme != FDLBM_SCHEME_T2S2_1 || o->precision != FDLBM_FP32_DEV || path != FDLBM_PATH_FUSED ||
@@ -154,10 +167,16 @@ bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
     const double nodes = (double)g->nx * g->ny;
     const bool warp = fused_warp_ok(g->nx, g->ny, g->bc_x == FDLBM_WALL);
     if (walled(g)) return !warp || nodes < tile_walled_nodes(o, false);
-    if (!warp) return nodes < 1.2e6;
     int tx, ty;
     tile_counts(g->nx, g->ny, false, false, &tx, &ty);
-    return nodes < (o->has_force ? 1.2e6 : 0.8e6) && nodes >= 0.7 * 512.0 * tx * ty;
+    const double tiled = 512.0 * tx * ty;
+    if (!warp) {
+        const int W = fused_tile_width();
+        const double swept = (double)((g->nx + W - 1) / W) * W * g->ny;
+        return nodes < 1.2e6 && tiled < 0.415e6 + 0.63 * swept;
+    }
+    if (nodes < 0.65 * tiled && std::max(g->nx, g->ny) > 4 * std::min(g->nx, g->ny)) return false;
+    return o->has_force ? nodes < 1.2e6 && tiled < 0.4e6 + 0.7 * nodes : nodes < 0.8e6 && tiled < 0.38e6 + 0.53 * nodes;
 }
 
 // Scratch fields a handle needs (see make_layout).
