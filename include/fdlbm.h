@@ -81,7 +81,8 @@ enum { FDLBM_EQ_STANDARD = 0, FDLBM_EQ_INCOMPRESSIBLE = 1 };
  * block through all stages in shared memory), where it is the fastest measured
  * on GB300: periodic grids under 0.8 M nodes (1.2 M with a force field, and
  * where WARP does not apply; not where a thin grid fills its tiles badly, or is
- * long and fills less than 0.65 of them), walled ones under 1.25 M (1.7 M with a force
+ * long and fills less than 0.65 of them), walled ones under 1.25 M (1.5 x 2^20 where a side has fewer
+ * than 256 nodes, 1.7 M with a force
  * field, any size where WARP does not apply).  Beyond that it picks WARP where
  * it applies, on a walled grid with the frame on the tile kernel (T2S2-FDLBM1),
  * and SCALAR otherwise; with path FUSED or a tile height given, WARP

@@ -108,11 +108,25 @@ bool use_split(const fdlbm_grid *g, const fdlbm_opts *o, int path)
 
 // Walled FP32 grids of fewer nodes run on the tile kernel rather than on the
 // warp tile and its frame (see use_tile; in a batch the frame is a walls sweep,
-// whose fixed cost is higher).
-double tile_walled_nodes(const fdlbm_opts *o, bool batch)
+// whose fixed cost is higher).  Thin ones are mostly frame: 66 x 20000 63.7 us
+// per step on the tile kernel, 102 on the warp tile with its frame, 88 on the walls
+// sweep; 20000 x 66 45 / 56 / 59.
+double tile_walled_nodes(const fdlbm_grid *g, const fdlbm_opts *o, bool batch)
 {
     if (batch) return o->has_force ? 4.0e6 : 2.4e6;
-    return o->has_force ? 1.7e6 : 1.25e6;
+    if (o->has_force) return 1.7e6;
+    return std::min(g->nx, g->ny) < 256 ? 1.5 * 1048576 : 1.25e6;
+}
+
+// The frame of a walled grid around the warp tile's interior (T2S2-FDLBM1): on the
+// tile kernel, except on channels of few rows, where the frame's tiles are a large
+// part of all (walls in y only, us per step, tile kernel against walls sweep:
+// 40000 x 66 105 / 81, 20000 x 161 80 / 77, 16000 x 200 71 / 73; with a force
+// field 40000 x 97 148 / 142, 20000 x 113 94 / 95).
+bool use_tile_frame(const fdlbm_grid *g, const fdlbm_opts *o)
+{
+    if (!walled(g) || o->scheme != FDLBM_SCHEME_T2S2_1 || o->variant != FDLBM_VARIANT_AUTO) return false;
+    return g->bc_x == FDLBM_WALL || g->ny >= (o->has_force ? 112 : 180);
 }
 
 // Walled T2S2-FDLBM2 grids (FP32) of fewer nodes run on the walls sweep rather
@@ -166,7 +180,7 @@ bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
         return false;
     const double nodes = (double)g->nx * g->ny;
     const bool warp = fused_warp_ok(g->nx, g->ny, g->bc_x == FDLBM_WALL);
-    if (walled(g)) return !warp || nodes < tile_walled_nodes(o, false);
+    if (walled(g)) return !warp || nodes < tile_walled_nodes(g, o, false);
     int tx, ty;
     tile_counts(g->nx, g->ny, false, false, &tx, &ty);
     const double tiled = 512.0 * tx * ty;
@@ -570,7 +584,7 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     // (2049^2 cavity 164 us per step against 95 on the warp tile)
     const bool auto_all = o.path == FDLBM_PATH_AUTO && o.rows_per_cta == 0;
     const double small_nodes = !s1                        ? warp_walled_nodes_s2(g)
-                               : force_staged || auto_all ? tile_walled_nodes(&o, force_staged)
+                               : force_staged || auto_all ? tile_walled_nodes(g, &o, force_staged)
                                                           : 1.5 * 1048576;
     const bool small_walled = walled(g) && (double)g->nx * g->ny < small_nodes;
     if (variant == FDLBM_VARIANT_AUTO)
@@ -622,7 +636,7 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     h->graph_steps = o.graph_steps > 0 ? o.graph_steps + (o.graph_steps & 1) : 0;
     h->split = !force_staged && use_split(g, &o, path);
     h->tile = !force_staged && use_tile(g, &o, path);
-    h->tile_frame = !force_staged && walled(g) && s1 && o.variant == FDLBM_VARIANT_AUTO;
+    h->tile_frame = !force_staged && use_tile_frame(g, &o);
     h->lay = make_layout(h->nx, h->ny, h->pitch, h->precision, h->has_force,
                          scratch_fields(g, &o, path, force_staged), h->split);
     cudaGetDevice(&h->device);
