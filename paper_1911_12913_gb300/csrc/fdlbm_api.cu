@@ -11,6 +11,7 @@
 #include <vector>
 
 #include "internal.h"
+#include "split_tables.h"
 
 using namespace fdlbm;
 
@@ -277,7 +278,8 @@ cudaError_t launch_split_steps(fdlbm_ctx *h, int n, cudaStream_t s)
     const bool walls = h->bc_x == FDLBM_WALL || h->bc_y == FDLBM_WALL;
     double *q0 = reinterpret_cast<double *>(h->ws + h->lay.Q);
     double *q1 = walls ? reinterpret_cast<double *>(h->ws + h->lay.P) : q0;
-    return launch_split(step_args<double>(h), q0, q1, reinterpret_cast<const double *>(h->ws + h->lay.split), n, s);
+    return launch_split(step_args<double>(h), q0, q1, reinterpret_cast<const double *>(h->ws + h->lay.split),
+                        h->split_merge, n, s);
 }
 
 // One step of whichever kernel the handle uses, reading state[cur], on stream s.
@@ -648,6 +650,7 @@ static cudaError_t upload_split_tables(fdlbm_ctx *h, const std::vector<double> &
 {
     const std::vector<double> t = make_split_tables(mx, my, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, h->beta,
                                                     h->A * h->dt, h->dt);
+    h->split_merge = split_centres_merge(t, h->nx, h->ny);
     return cudaMemcpy(h->ws + h->lay.split, t.data(), t.size() * sizeof(double), cudaMemcpyHostToDevice);
 }
 

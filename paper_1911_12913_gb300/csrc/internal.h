@@ -78,6 +78,7 @@ struct fdlbm_ctx {
     bool in_batch = false;               // owned by a batch: stepped by fdlbm_batch_step
     bool adjoint = false;                // scratch for the adjoint step reserved
     bool split = false;                  // two launches per step (step_split.cu), in place
+    bool split_merge = false;            // the centre weights of its diagonals merge exactly
     bool uniform = false;                // one metric value on each axis
     bool tile_frame = false;             // warp tile: the frame on the tile kernel
     bool tile = false;                   // FP32 tile kernel (step_tile.cu)
@@ -183,10 +184,8 @@ int fused_tile_width_walls();
 // step_split.cu (FP64, two launches per step, one node per thread; the state in
 // s.gin is advanced in place, s.gout is scratch)
 size_t split_table_bytes(int nx, int ny);
-std::vector<double> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
-                                      double beta, double h, double dt);
-cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, int nsteps,
-                         cudaStream_t stream);
+cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, bool merge,
+                         int nsteps, cudaStream_t stream);  // merge: split_centres_merge of the tables
 // step_tile.cu (FP32 T2S2-FDLBM1, one launch per step, a tile per block)
 void tile_counts(int nx, int ny, bool wall_x, bool wall_y, int *tx, int *ty);
 int tile_launches(int nx, int ny, bool wall_x, bool wall_y);  // of one step

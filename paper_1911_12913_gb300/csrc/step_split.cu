@@ -14,9 +14,11 @@
 // node, so on walled grids Q alternates between two buffers.
 //
 // The difference weights come from tables with the metric, the time step and
-// the sign folded in (make_split_tables): one multiply-add per tap, and next to
+// the sign folded in (split_tables.h): one multiply-add per tap, and next to
 // a wall, where the second-order upwind tap would leave the domain, the entry
-// of that sign holds the central difference.
+// of that sign holds the central difference.  The weights of each axis sum to
+// exactly zero, and stay so in the kernels: the centre weights of a diagonal are
+// added into one only where that sum is exact (MERGE: uniform periodic grids).
 //
 // What bounds it: the FP64 units, 227 FP64 instructions per node (prepare
 // 79, star 104, update 44): 1024^2 periodic 431 us per step, 0.87 of the rate at
@@ -33,6 +35,7 @@
 
 #include "chain.cuh"
 #include "internal.h"
+#include "split_tables.h"
 #include "walls_nodes.cuh"
 
 namespace fdlbm {
@@ -82,7 +85,7 @@ __device__ __forceinline__ Taps<R> load_taps(const R *t)
 
 // A node, its neighbours (wrapped on a periodic axis; on a walled axis clamped,
 // where the weights are zero) and the weights of its differences.
-template <class R, bool WALLS>
+template <class R, bool WALLS, bool MERGE>
 struct Site {
     int x[5], y[5];          // k - 2 .. k + 2
     Taps<R> xp, xn, yp, yn;  // weights for the signs of each axis
@@ -109,10 +112,11 @@ struct Site {
     __device__ __forceinline__ R advance(const R *f, int i, R v0, R acc) const
     {
         const int r0 = y[2];
-        // one multiply-add per tap, the centre weights of a diagonal merged
-        if (cx(i) != 0 && cy(i) != 0) acc = fma((cx(i) > 0 ? xp.c : xn.c) + (cy(i) > 0 ? yp.c : yn.c), v0, acc);
-        else if (cx(i) != 0) acc = fma(cx(i) > 0 ? xp.c : xn.c, v0, acc);
-        else acc = fma(cy(i) > 0 ? yp.c : yn.c, v0, acc);
+        if (MERGE && cx(i) != 0 && cy(i) != 0) acc = fma(xp.c + yp.c, v0, acc);
+        else {
+            if (cx(i) != 0) acc = fma(cx(i) > 0 ? xp.c : xn.c, v0, acc);
+            if (cy(i) != 0) acc = fma(cy(i) > 0 ? yp.c : yn.c, v0, acc);
+        }
         if (cx(i) != 0) {
             const Taps<R> &w = cx(i) > 0 ? xp : xn;
             const int s = cx(i);
@@ -308,12 +312,13 @@ __device__ __forceinline__ void load_force(const SplitArgs<R> &a, int x, int y, 
 // shuffles: those past the last node work on a copy of the first.  (129^2 cavity,
 // whose wall nodes alone are split: 20.9 -> 14.2 us per step; 64^2 periodic 11.6 ->
 // 7.1.)
-template <class R, bool FORCE>
+template <class R, bool FORCE, bool MERGE>
 struct Quad {
     const SplitArgs<R> &a;
     const int q;
     const R ax, ay, dx, dy;  // velocities
     Taps<R> wx, wy;
+    R wxy;                   // MERGE: the centre weight of the diagonal population
     int o0, x[3], y[3];      // offsets at k, and at k + s, k - s, k - 2s in x and in y
     R drho, jx, jy, rm, inv, h45, base;
 
@@ -341,6 +346,7 @@ struct Quad {
         }
         wx = load_taps(a.tx + 8 * xc + (sx > 0 ? 0 : 4));
         wy = load_taps(a.ty + 8 * yc + (sy > 0 ? 0 : 4));
+        if (MERGE) wxy = wx.c + wy.c;
     }
 
     // acc plus the weighted taps of the axis and of the diagonal population
@@ -354,7 +360,9 @@ struct Quad {
     }
     __device__ __forceinline__ R diagonal(const R *f, R acc) const
     {
-        acc = fma(wx.c + wy.c, f[o0], acc);
+        const R v0 = f[o0];
+        if (MERGE) acc = fma(wxy, v0, acc);
+        else acc = fma(wy.c, v0, fma(wx.c, v0, acc));
         acc = fma(wx.m1, f[x[0]], acc);
         acc = fma(wy.m1, f[y[0]], acc);
         acc = fma(wx.p1, f[x[1]], acc);
@@ -414,7 +422,7 @@ struct Quad {
     }
 };
 
-template <class R, bool FORCE, bool WALLS>
+template <class R, bool FORCE, bool WALLS, bool MERGE>
 __device__ __forceinline__ void star_quad(const SplitArgs<R> &a)
 {
     int x, y;
@@ -426,7 +434,7 @@ __device__ __forceinline__ void star_quad(const SplitArgs<R> &a)
     }
     int jx = x, jy = y, side = -1;
     if (WALLS) side = wall_side(a, x, y, jx, jy);  // a wall for the whole block, or for none of it
-    Quad<R, FORCE> n(a);
+    Quad<R, FORCE, MERGE> n(a);
     n.set(jx, jy);
     R Fx, Fy;
     load_force<R, FORCE>(a, jx, jy, Fx, Fy);
@@ -455,7 +463,7 @@ __device__ __forceinline__ void star_quad(const SplitArgs<R> &a)
     a.S[pd + o] = gd;
 }
 
-template <class R, bool FORCE, bool WALLS, bool LAST>
+template <class R, bool FORCE, bool WALLS, bool MERGE, bool LAST>
 __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
 {
     int x, y;
@@ -467,7 +475,7 @@ __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
     }
     int jx = x, jy = y, side = -1;
     if (WALLS) side = wall_side(a, x, y, jx, jy);
-    Quad<R, FORCE> n(a);
+    Quad<R, FORCE, MERGE> n(a);
     n.set(jx, jy);
     chain_wait();
     const size_t pa = (1 + n.q) * a.plane, pd = (5 + n.q) * a.plane;
@@ -535,18 +543,18 @@ __global__ void __launch_bounds__(kThreads) k_split_prepare(const SplitArgs<R> a
 }
 
 // QUAD: four threads per node for every node; else for the wall nodes.
-template <class R, bool FORCE, bool WALLS, bool QUAD>
+template <class R, bool FORCE, bool WALLS, bool QUAD, bool MERGE>
 __global__ void __launch_bounds__(kThreads) k_split_star(const SplitArgs<R> a)
 {
     if (QUAD || (WALLS && blockIdx.x < a.wall_blocks)) {
-        star_quad<R, FORCE, WALLS>(a);
+        star_quad<R, FORCE, WALLS, MERGE>(a);
         return;
     }
     int x, y;
     if (!my_node<R, WALLS>(a, x, y)) return;
     int jx = x, jy = y, side = -1;
     if (WALLS) side = wall_side(a, x, y, jx, jy);
-    Site<R, WALLS> n;
+    Site<R, WALLS, MERGE> n;
     n.set(a, jx, jy);
     R Fx, Fy;
     load_force<R, FORCE>(a, jx, jy, Fx, Fy);
@@ -572,18 +580,18 @@ __global__ void __launch_bounds__(kThreads) k_split_star(const SplitArgs<R> a)
     for (int i = 1; i < 9; ++i) a.S[i * a.plane + o] = st[i];
 }
 
-template <class R, bool FORCE, bool WALLS, bool QUAD, bool LAST>
+template <class R, bool FORCE, bool WALLS, bool QUAD, bool MERGE, bool LAST>
 __global__ void __launch_bounds__(kThreads) k_split_update(const SplitArgs<R> a)
 {
     if (QUAD || (WALLS && blockIdx.x < a.wall_blocks)) {
-        update_quad<R, FORCE, WALLS, LAST>(a);
+        update_quad<R, FORCE, WALLS, MERGE, LAST>(a);
         return;
     }
     int x, y;
     if (!my_node<R, WALLS>(a, x, y)) return;
     int jx = x, jy = y, side = -1;
     if (WALLS) side = wall_side(a, x, y, jx, jy);
-    Site<R, WALLS> n;
+    Site<R, WALLS, MERGE> n;
     n.set(a, jx, jy);
     chain_wait();
     R g[9];
@@ -643,7 +651,7 @@ cudaError_t launch(K kernel, SplitArgs<R> a, int lanes, bool split_walls, bool c
     return cudaGetLastError();
 }
 
-template <class R, bool FORCE, bool WALLS, bool QUAD>
+template <class R, bool FORCE, bool WALLS, bool QUAD, bool MERGE>
 cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStream_t s)
 {
     const R *bx = tabs, *by = tabs + 8 * (size_t)a.nx;                     // stage B (scale -h m)
@@ -655,58 +663,21 @@ cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStr
         const bool last = k + 1 == nsteps;
         a.tx = bx;
         a.ty = by;
-        e = launch<R>(k_split_star<R, FORCE, WALLS, QUAD>, a, QUAD ? 4 : 1, WALLS, true, s);
+        e = launch<R>(k_split_star<R, FORCE, WALLS, QUAD, MERGE>, a, QUAD ? 4 : 1, WALLS, true, s);
         if (e != cudaSuccess) break;
         a.tx = cxs;
         a.ty = cys;
         a.Qin = q[k & 1];
         a.Qout = last ? a.P : q[(k + 1) & 1];
-        e = last ? launch<R>(k_split_update<R, FORCE, WALLS, QUAD, true>, a, QUAD ? 4 : 1, WALLS, true, s)
-                 : launch<R>(k_split_update<R, FORCE, WALLS, QUAD, false>, a, QUAD ? 4 : 1, WALLS, true, s);
+        e = last ? launch<R>(k_split_update<R, FORCE, WALLS, QUAD, MERGE, true>, a, QUAD ? 4 : 1, WALLS, true, s)
+                 : launch<R>(k_split_update<R, FORCE, WALLS, QUAD, MERGE, false>, a, QUAD ? 4 : 1, WALLS, true, s);
     }
     return e;
-}
-
-// Weights of the mixed difference at one node of an axis, times `scale`, for
-// velocity sign +1 or -1: {k + s, k, k - s, k - 2s}; `central`: next to a wall.
-void taps(const Stencil<double> &st, bool central, double scale, double out[4])
-{
-    const double m1 = scale * (central ? 0.5 : st.wm1), p1 = scale * (central ? -0.5 : st.w1);
-    const double p2 = scale * (central ? 0.0 : st.w2);
-    out[0] = m1;
-    out[1] = -((m1 + p1) + p2);
-    out[2] = p1;
-    out[3] = p2;
 }
 
 }  // namespace
 
 size_t split_table_bytes(int nx, int ny) { return 16 * (size_t)(nx + ny) * sizeof(double); }
-
-// The tables in the order bx, by, cx, cy: [n][2][4] each.
-std::vector<double> make_split_tables(const std::vector<double> &mx, const std::vector<double> &my, bool wx, bool wy,
-                                      double beta, double h, double dt)
-{
-    const Stencil<double> st = make_stencil<double>(beta);
-    std::vector<double> out;
-    out.reserve(16 * (mx.size() + my.size()));
-    auto axis = [&](const std::vector<double> &m, bool wall, double s) {
-        const int n = (int)m.size();
-        for (int k = 0; k < n; ++k)
-            for (int sign = 1; sign >= -1; sign -= 2) {
-                // the second-order upwind tap k - 2 s would leave the domain
-                const bool central = wall && (sign > 0 ? k < 2 : k > n - 3);
-                double t[4];
-                taps(st, central, -s * m[k], t);
-                out.insert(out.end(), t, t + 4);
-            }
-    };
-    axis(mx, wx, h);
-    axis(my, wy, h);
-    axis(mx, wx, dt);
-    axis(my, wy, dt);
-    return out;
-}
 
 // Grids of at most so many nodes take four threads per node throughout: up to two
 // such warps per scheduler of 152 SMs on a periodic grid, one on a walled one
@@ -715,8 +686,8 @@ std::vector<double> make_split_tables(const std::vector<double> &mx, const std::
 constexpr long long kQuadNodes = 9728, kQuadWalledNodes = 4864;
 
 // nsteps steps of the state in s.gin, in place.
-cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, int nsteps,
-                         cudaStream_t stream)
+cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, const double *tables, bool merge,
+                         int nsteps, cudaStream_t stream)
 {
     using R = double;
     if (nsteps <= 0) return cudaSuccess;
@@ -740,18 +711,17 @@ cudaError_t launch_split(const StepArgs<double> &s, double *Q0, double *Q1, cons
     a.l_star[0] = s.c.b_star * LinearCoef<R>::c1;
     a.l_star[1] = s.c.b_star * LinearCoef<R>::c2;
     const bool walls = a.wx || a.wy;
-    auto go = [&](auto force, auto wl, auto quad) {
-        constexpr bool F = decltype(force)::value, W = decltype(wl)::value, Q = decltype(quad)::value;
-        return run<R, F, W, Q>(a, Q0, Q1, tables, nsteps, stream);
+    const std::true_type y{};
+    const std::false_type n{};
+    auto go = [&](auto wl, auto quad, auto mg) {
+        constexpr bool W = decltype(wl)::value, Q = decltype(quad)::value, M = decltype(mg)::value;
+        return s.force ? run<R, true, W, Q, M>(a, Q0, Q1, tables, nsteps, stream)
+                       : run<R, false, W, Q, M>(a, Q0, Q1, tables, nsteps, stream);
     };
-    auto pick = [&](auto quad) {
-        const std::true_type y{};
-        const std::false_type n{};
-        if (walls) return s.force ? go(y, y, quad) : go(n, y, quad);
-        return s.force ? go(y, n, quad) : go(n, n, quad);
-    };
-    if ((long long)a.nx * a.ny <= (walls ? kQuadWalledNodes : kQuadNodes)) return pick(std::true_type{});
-    return pick(std::false_type{});
+    const bool quad = (long long)a.nx * a.ny <= (walls ? kQuadWalledNodes : kQuadNodes);
+    if (walls) return quad ? go(y, y, n) : go(y, n, n);
+    if (quad) return merge ? go(n, y, y) : go(n, y, n);
+    return merge ? go(n, n, y) : go(n, n, n);
 }
 
 }  // namespace fdlbm
