@@ -13,8 +13,9 @@ namespace fdlbm {
 // Two identities of the exact weights hold for the rounded ones, because an error
 // in them adds up over the steps: the sum is zero (else every step scales the
 // population), and the difference of a linear function is `scale` times its slope
-// (else populations travel at another speed: taps rounded one by one, 192^2 Taylor
-// vortex in a mean flow after 1000 steps 8e-15 off in the momentum, 7e-16 so).
+// (else populations travel at another speed: taps rounded one by one, 64^2 Taylor
+// vortex in a mean flow after 1000 steps, momentum 1.6e-15 off 80-bit arithmetic,
+// 9e-16 so).
 // All weights are multiples of q = 2^(e - 52), 2^e <= |scale| < 2^(e + 1), or of 2q
 // for a blend above 0.3, where they may exceed |scale|: then every sum below is at
 // most 2^53 q and exact.
