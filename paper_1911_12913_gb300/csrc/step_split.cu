@@ -515,6 +515,9 @@ __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
     relax(g0, e0, f0, P0, Q0);
     relax(ga, ea, fa, Pa, Qa);
     relax(gd, ed, fd, Pd, Qd);
+    // on a periodic grid Qout is Qin: all four threads have read the rest population
+    // that one of them now writes (a shuffle orders no memory)
+    __syncwarp();
     chain_next();
     if (!valid) return;
     if (n.q == 0) {
