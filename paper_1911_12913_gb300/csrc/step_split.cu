@@ -467,6 +467,46 @@ __device__ __forceinline__ void star_quad(const SplitArgs<R> &a)
     a.S[pd + o] = gd;
 }
 
+// P and Q of node o from its f~, four threads per node.  The first launch of a call
+// and the update both come here (and to prepare), so that a state does not depend
+// on how its steps are divided into calls.
+template <class R, bool FORCE, bool MERGE>
+__device__ __forceinline__ void prepare_quad(const SplitArgs<R> &a, Quad<R, FORCE, MERGE> &n, size_t o, bool valid, R g0,
+                                             R ga, R gd, R Fx, R Fy)
+{
+    const size_t pa = (1 + n.q) * a.plane, pd = (5 + n.q) * a.plane;
+    n.macro(g0, ga, gd, Fx, Fy, a.c.half_dt);
+    R e0, ea, ed, f0 = R(0), fa = R(0), fd = R(0);
+    n.equilibrium(e0, ea, ed);
+    if (FORCE) n.force_term(e0, ea, ed, Fx, Fy, f0, fa, fd);
+    auto relax = [&](R g, R e, R f, R &P, R &Q) {
+        const R neq = e - g;
+        P = fma(a.c.b_bar, neq, g);
+        Q = fma(a.c.b_til, neq, g);
+        if (FORCE) {
+            P = fma(a.c.c_bar, f, P);
+            Q = fma(a.c.c_til, f, Q);
+        }
+    };
+    R P0, Q0, Pa, Qa, Pd, Qd;
+    relax(g0, e0, f0, P0, Q0);
+    relax(ga, ea, fa, Pa, Qa);
+    relax(gd, ed, fd, Pd, Qd);
+    // P lies over f~, and on a periodic grid Qout is Qin: all four threads have read
+    // the rest population that one of them now writes (a shuffle orders no memory)
+    __syncwarp();
+    chain_next();
+    if (!valid) return;
+    if (n.q == 0) {
+        a.P[o] = P0;
+        a.Qout[o] = Q0;
+    }
+    a.P[pa + o] = Pa;
+    a.P[pd + o] = Pd;
+    a.Qout[pa + o] = Qa;
+    a.Qout[pd + o] = Qd;
+}
+
 template <class R, bool FORCE, bool WALLS, bool MERGE, bool LAST>
 __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
 {
@@ -498,45 +538,29 @@ __device__ __forceinline__ void update_quad(const SplitArgs<R> &a)
         return;
     }
     load_force<R, FORCE>(a, x, y, Fx, Fy);
-    n.macro(g0, ga, gd, Fx, Fy, a.c.half_dt);
-    R e0, ea, ed, f0 = R(0), fa = R(0), fd = R(0);
-    n.equilibrium(e0, ea, ed);
-    if (FORCE) n.force_term(e0, ea, ed, Fx, Fy, f0, fa, fd);
-    auto relax = [&](R g, R e, R f, R &P, R &Q) {
-        const R neq = e - g;
-        P = fma(a.c.b_bar, neq, g);
-        Q = fma(a.c.b_til, neq, g);
-        if (FORCE) {
-            P = fma(a.c.c_bar, f, P);
-            Q = fma(a.c.c_til, f, Q);
-        }
-    };
-    R P0, Q0, Pa, Qa, Pd, Qd;
-    relax(g0, e0, f0, P0, Q0);
-    relax(ga, ea, fa, Pa, Qa);
-    relax(gd, ed, fd, Pd, Qd);
-    // on a periodic grid Qout is Qin: all four threads have read the rest population
-    // that one of them now writes (a shuffle orders no memory)
-    __syncwarp();
-    chain_next();
-    if (!valid) return;
-    if (n.q == 0) {
-        a.P[o] = P0;
-        a.Qout[o] = Q0;
-    }
-    a.P[pa + o] = Pa;
-    a.P[pd + o] = Pd;
-    a.Qout[pa + o] = Qa;
-    a.Qout[pd + o] = Qd;
+    prepare_quad<R, FORCE, MERGE>(a, n, o, valid, g0, ga, gd, Fx, Fy);
 }
 
-template <class R, bool FORCE>
+// QUAD, here and below: four threads per node for every node; else for the wall
+// nodes.
+template <class R, bool FORCE, bool WALLS, bool QUAD>
 __global__ void __launch_bounds__(kThreads) k_split_prepare(const SplitArgs<R> a)
 {
     int x, y;
-    if (!my_node<R, false>(a, x, y)) return;
+    R Fx, Fy;
+    if (QUAD || (WALLS && blockIdx.x < a.wall_blocks)) {
+        const bool valid = my_node<R, WALLS, 4>(a, x, y);
+        if (!valid) x = y = 0;
+        const size_t o = (size_t)y * a.pitch + x;
+        Quad<R, FORCE, false> n(a);
+        load_force<R, FORCE>(a, x, y, Fx, Fy);
+        prepare_quad<R, FORCE, false>(a, n, o, valid, a.P[o], a.P[(1 + n.q) * a.plane + o],
+                                      a.P[(5 + n.q) * a.plane + o], Fx, Fy);
+        return;
+    }
+    if (!my_node<R, WALLS>(a, x, y)) return;
     const size_t o = (size_t)y * a.pitch + x;
-    R g[9], P[9], Q[9], Fx, Fy;
+    R g[9], P[9], Q[9];
 #pragma unroll
     for (int i = 0; i < 9; ++i) g[i] = a.P[i * a.plane + o];
     load_force<R, FORCE>(a, x, y, Fx, Fy);
@@ -549,7 +573,6 @@ __global__ void __launch_bounds__(kThreads) k_split_prepare(const SplitArgs<R> a
     }
 }
 
-// QUAD: four threads per node for every node; else for the wall nodes.
 template <class R, bool FORCE, bool WALLS, bool QUAD, bool MERGE>
 __global__ void __launch_bounds__(kThreads) k_split_star(const SplitArgs<R> a)
 {
@@ -665,7 +688,7 @@ cudaError_t run(SplitArgs<R> a, R *Q0, R *Q1, const R *tabs, int nsteps, cudaStr
     const R *cxs = by + 8 * (size_t)a.ny, *cys = cxs + 8 * (size_t)a.nx;   // stage C (scale -dt m)
     R *q[2] = {Q0, Q1};
     a.Qout = q[0];
-    cudaError_t e = launch<R>(k_split_prepare<R, FORCE>, a, 1, false, false, s);
+    cudaError_t e = launch<R>(k_split_prepare<R, FORCE, WALLS, QUAD>, a, QUAD ? 4 : 1, WALLS, false, s);
     for (int k = 0; k < nsteps && e == cudaSuccess; ++k) {
         const bool last = k + 1 == nsteps;
         a.tx = bx;

@@ -1,5 +1,7 @@
 """Bits of the FP64 split step: the same from run to run, where four threads of a
-node read what one of them then overwrites in place."""
+node read what one of them then overwrites in place; and the same however the
+steps are divided into calls or replayed from a graph, so that a run can be
+stopped and resumed."""
 import numpy as np
 import pytest
 
@@ -37,3 +39,23 @@ def _solver(x, y, nx, ny, force, **kw):
 def test_in_place_quads_give_the_same_bits_every_time(nx, ny, force):
     states = [_solver("periodic", "periodic", nx, ny, force).step(100).get_state() for _ in range(3)]
     assert np.array_equal(states[0], states[1]) and np.array_equal(states[0], states[2])
+
+
+@pytest.mark.parametrize("x,y,nx,ny,force", [
+    ("periodic", "periodic", 64, 64, False), ("periodic", "periodic", 33, 17, True),
+    ("periodic", "periodic", 160, 129, False), ("periodic", "periodic", 160, 129, True),
+    ("wall", "wall", 33, 33, False), ("wall", "wall", 40, 30, True), ("wall", "wall", 129, 97, False),
+    ("wall", "wall", 129, 97, True), ("periodic", "wall", 150, 70, True), ("wall", "periodic", 150, 70, False),
+])
+def test_state_does_not_depend_on_the_division_into_calls(x, y, nx, ny, force):
+    whole = _solver(x, y, nx, ny, force).step(24).get_state()
+    s = _solver(x, y, nx, ny, force)
+    for n in (1, 1, 2, 5, 1, 14):
+        s.step(n)
+    assert np.array_equal(s.get_state(), whole)
+    assert np.array_equal(_solver(x, y, nx, ny, force, graph_steps=4).step(24).get_state(), whole)
+    # resumed from a saved state
+    s = _solver(x, y, nx, ny, force).step(10)
+    kept = s.save_state(s.new_buffer())
+    s.step(3)
+    assert np.array_equal(s.load_state(kept).step(14).get_state(), whole)
