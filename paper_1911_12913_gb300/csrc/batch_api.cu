@@ -286,7 +286,8 @@ bool uses_fused_sweep(const fdlbm_batch_ctx *b)
 // Tile height of the fused batch's sweeps: minimise (waves) x (rows + 8) over the
 // tiles of all cases, as for a single grid, with the waves of the warp-tile
 // launches and of the scalar sweeps counted separately (they run one after the
-// other).  In FUSED mode the tile kernel's cases have no say.
+// other).  In FUSED mode the tile kernel's cases have no say; where there are no
+// others, no height is better than another and the first one stands.
 int fused_rows_model(const fdlbm_batch_ctx *b)
 {
     int dev = 0, sms = 152;
@@ -308,6 +309,7 @@ int fused_rows_model(const fdlbm_batch_ctx *b)
             else if (!fused || !s1)
                 ctas += (long long)((h->nx + W - 1) / W) * ty;
         }
+        if (ctas + wtiles == 0) break;
         const double cost = (double)((ctas + slots - 1) / slots + (wtiles + wslots - 1) / wslots) * (rows + 8);
         if (cost < best_cost - 1e-9) {
             best_cost = cost;
@@ -410,12 +412,14 @@ fdlbm_status capture(fdlbm_batch_ctx *b)
     return FDLBM_OK;
 }
 
+// What the choice depends on: the mode, and each case's grid and kernel instance.
 std::string signature(const fdlbm_batch_ctx *b)
 {
     std::ostringstream os;
     os << b->precision << '/' << b->mode;
     for (const fdlbm_ctx *h : b->cases)
-        os << ';' << h->nx << 'x' << h->ny << ':' << h->bc_x << h->bc_y << h->has_force << h->scheme;
+        os << ';' << h->nx << 'x' << h->ny << ':' << h->bc_x << h->bc_y << h->has_force << h->scheme << h->incomp
+           << (h->variant == FDLBM_VARIANT_WARP);
     return os.str();
 }
 
