@@ -142,7 +142,7 @@ typedef struct {
     int rows_per_cta;         /* fused kernel tile height; 0 = automatic */
     int variant;              /* FDLBM_VARIANT_*; WARP where it does not apply -> EUNSUPPORTED */
     int scheme;               /* FDLBM_SCHEME_T2S2_1 (default) or FDLBM_SCHEME_T2S2_2 */
-    int adjoint;              /* 1: reserve scratch for fdlbm_adjoint_step (periodic grids) */
+    int adjoint;              /* 1: fdlbm_adjoint_step may be called (periodic grids) */
     int graph_steps;          /* > 0: fdlbm_step replays a CUDA graph of this many steps (rounded
                                  up to even), captured on first use; 0 = direct launches */
     int equilibrium;          /* FDLBM_EQ_STANDARD (Eq. 3.2) or FDLBM_EQ_INCOMPRESSIBLE */

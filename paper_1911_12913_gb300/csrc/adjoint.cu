@@ -461,8 +461,7 @@ template cudaError_t launch_init_vjp<double>(const StepArgs<double> &, const dou
                                              double *, double *, double *, double *, cudaStream_t);
 
 template <class R>
-cudaError_t launch_adjoint(const StepArgs<R> &a, const R *lam_next, R *lam_prev, R *, R *,
-                           double *, double *dforce, cudaStream_t s)
+cudaError_t launch_adjoint(const StepArgs<R> &a, const R *lam_next, R *lam_prev, double *dforce, cudaStream_t s)
 {
     const bool force = a.force != nullptr;
     AdjArgs<R> p{a, lam_next, lam_prev, dforce, adj_rows(a.nx, a.ny, adj_blocks_per_sm<R>(force))};
@@ -485,10 +484,9 @@ cudaError_t launch_moments_vjp(const StepArgs<R> &a, const double *du, R *lam, d
     return cudaGetLastError();
 }
 
-template cudaError_t launch_adjoint<float>(const StepArgs<float> &, const float *, float *, float *,
-                                           float *, double *, double *, cudaStream_t);
-template cudaError_t launch_adjoint<double>(const StepArgs<double> &, const double *, double *,
-                                            double *, double *, double *, double *, cudaStream_t);
+template cudaError_t launch_adjoint<float>(const StepArgs<float> &, const float *, float *, double *, cudaStream_t);
+template cudaError_t launch_adjoint<double>(const StepArgs<double> &, const double *, double *, double *,
+                                            cudaStream_t);
 template cudaError_t launch_moments_vjp<float>(const StepArgs<float> &, const double *, float *,
                                                double *, cudaStream_t);
 template cudaError_t launch_moments_vjp<double>(const StepArgs<double> &, const double *, double *,

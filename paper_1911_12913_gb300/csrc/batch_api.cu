@@ -540,8 +540,7 @@ size_t fdlbm_batch_workspace_bytes(int ncases, const fdlbm_grid *grids, const fd
         fdlbm_opts o;
         fdlbm_default_opts(&o);
         if (opts) o = opts[c];
-        o.path = FDLBM_PATH_STAGED;
-        const size_t s = fdlbm_workspace_bytes(&grids[c], &o);
+        const size_t s = handle_workspace_bytes(&grids[c], o, true);
         if (s == 0) return 0;
         total += align_b(s);
     }

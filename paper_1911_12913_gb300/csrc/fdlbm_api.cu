@@ -194,12 +194,13 @@ bool use_tile(const fdlbm_grid *g, const fdlbm_opts *o, int path)
     return o->has_force ? nodes < 1.2e6 && tiled < 0.4e6 + 0.7 * nodes : nodes < 0.8e6 && tiled < 0.38e6 + 0.53 * nodes;
 }
 
-// Scratch fields a handle needs (see make_layout).
+// Scratch fields a handle needs (see make_layout).  The split step comes first: it
+// also runs on the staged path, and makes f* in the other state buffer.  The
+// adjoint needs none.
 int scratch_fields(const fdlbm_grid *g, const fdlbm_opts *o, int path, bool force_staged)
 {
-    if (force_staged || path == FDLBM_PATH_STAGED || o->adjoint) return 3;
-    if (use_split(g, o, path)) return walled(g) ? 2 : 1;
-    return 0;
+    if (!force_staged && use_split(g, o, path)) return walled(g) ? 2 : 1;
+    return force_staged || path == FDLBM_PATH_STAGED ? 3 : 0;
 }
 
 // Rows per CTA of the fused kernel.  Each CTA recomputes 8 halo rows, so tall
@@ -646,6 +647,16 @@ fdlbm_status handle_prepare(const fdlbm_grid *g, const fdlbm_metrics *metrics, d
     return FDLBM_OK;
 }
 
+size_t handle_workspace_bytes(const fdlbm_grid *g, const fdlbm_opts &o, bool force_staged)
+{
+    if (!grid_ok(g)) return 0;
+    const int path = force_staged ? FDLBM_PATH_STAGED : choose_path(g, &o);
+    if (path < 0) return 0;
+    return make_layout(g->nx, g->ny, pitch_of(g->nx), o.precision, o.has_force,
+                       scratch_fields(g, &o, path, force_staged), !force_staged && use_split(g, &o, path))
+        .total;
+}
+
 static cudaError_t upload_split_tables(fdlbm_ctx *h, const std::vector<double> &mx, const std::vector<double> &my)
 {
     const std::vector<double> t = make_split_tables(mx, my, h->bc_x == FDLBM_WALL, h->bc_y == FDLBM_WALL, h->beta,
@@ -722,12 +733,7 @@ size_t fdlbm_workspace_bytes(const fdlbm_grid *g, const fdlbm_opts *opts)
     fdlbm_opts o;
     fdlbm_default_opts(&o);
     if (opts) o = *opts;
-    if (!grid_ok(g)) return 0;
-    const int path = choose_path(g, &o);
-    if (path < 0) return 0;
-    return make_layout(g->nx, g->ny, pitch_of(g->nx), o.precision, o.has_force,
-                       scratch_fields(g, &o, path, false), use_split(g, &o, path))
-        .total;
+    return handle_workspace_bytes(g, o, false);
 }
 
 fdlbm_status fdlbm_create(const fdlbm_grid *g, const fdlbm_metrics *metrics, double nu,
@@ -1013,7 +1019,6 @@ fdlbm_status fdlbm_adjoint_step(fdlbm_t h, const void *state_n, const void *lam_
         return fail(h, FDLBM_EUNSUPPORTED,
                     "adjoint_step: needs opts.adjoint, a periodic grid and scheme T2S2_1");
     cudaError_t e;
-    double *fB = reinterpret_cast<double *>(h->ws + h->lay.S);
     if (h->precision == FDLBM_FP32_DEV) {
         StepArgs<float> a = step_args<float>(h);
         a.gin = static_cast<const float *>(state_n);
@@ -1021,12 +1026,12 @@ fdlbm_status fdlbm_adjoint_step(fdlbm_t h, const void *state_n, const void *lam_
         float *lp = static_cast<float *>(lam_prev);
         e = adjoint_tile_ok(state_n, lam_next, lam_prev)
                 ? launch_adjoint_tile(a, h->uniform, ln, lp, dforce, h->stream)
-                : launch_adjoint<float>(a, ln, lp, a.P, a.Q, fB, dforce, h->stream);
+                : launch_adjoint<float>(a, ln, lp, dforce, h->stream);
     } else {
         StepArgs<double> a = step_args<double>(h);
         a.gin = static_cast<const double *>(state_n);
         e = launch_adjoint<double>(a, static_cast<const double *>(lam_next),
-                                   static_cast<double *>(lam_prev), a.P, a.Q, fB, dforce, h->stream);
+                                   static_cast<double *>(lam_prev), dforce, h->stream);
     }
     return e == cudaSuccess ? FDLBM_OK : cuda_fail(h, e, "adjoint_step");
 }

@@ -76,7 +76,7 @@ struct fdlbm_ctx {
     int path = FDLBM_PATH_FUSED;
     int variant = FDLBM_VARIANT_SCALAR;  // fused kernel actually used
     bool in_batch = false;               // owned by a batch: stepped by fdlbm_batch_step
-    bool adjoint = false;                // scratch for the adjoint step reserved
+    bool adjoint = false;                // fdlbm_adjoint_step allowed
     bool split = false;                  // two launches per step (step_split.cu), in place
     bool split_merge = false;            // the centre weights of its diagonals merge exactly
     bool uniform = false;                // one metric value on each axis
@@ -110,8 +110,9 @@ fdlbm_status handle_upload(fdlbm_ctx *h, const std::vector<double> &mx,
                            const std::vector<double> &my);
 template <class R>
 StepArgs<R> handle_step_args(fdlbm_ctx *h);
-// Scratch fields of a handle: all three (staged kernels, adjoint), or the f~+
-// buffers of the split step (two on walled grids), and the split step's tables.
+// Scratch fields of a handle: all three (staged kernels), or the f~+ buffers of the
+// split step (two on walled grids), and the split step's tables.
+size_t handle_workspace_bytes(const fdlbm_grid *g, const fdlbm_opts &o, bool force_staged);
 Layout make_layout(int nx, int ny, int pitch, int precision, int has_force, int scratch, bool split);
 
 // step_fused.cu
@@ -217,8 +218,7 @@ cudaError_t launch_adjoint_tile(const StepArgs<float> &a, bool uniform, const fl
                                 double *dforce, cudaStream_t s);
 // adjoint.cu
 template <class R>
-cudaError_t launch_adjoint(const StepArgs<R> &a, const R *lam_next, R *lam_prev, R *P, R *lgs,
-                           double *fB, double *dforce, cudaStream_t s);
+cudaError_t launch_adjoint(const StepArgs<R> &a, const R *lam_next, R *lam_prev, double *dforce, cudaStream_t s);
 template <class R>
 cudaError_t launch_init_vjp(const StepArgs<R> &a, const double *rho, const double *ux,
                             const double *uy, const R *lam, double dt, double *drho, double *dux,
