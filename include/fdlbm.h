@@ -76,20 +76,20 @@ enum { FDLBM_EQ_STANDARD = 0, FDLBM_EQ_INCOMPRESSIBLE = 1 };
  *          (there the walled and the periodic scheme compute the same values),
  *          and a second launch of the walls sweep covers the 4-node frame:
  *          two launches per step (fdlbm_kernels_per_step).
- * AUTO (with path AUTO and rows_per_cta 0) runs FP32 grids of small and medium
- * size on the tile kernel (one launch per step, a tile of 32 x 16 nodes per
- * block through all stages in shared memory), where it is the fastest measured
- * on GB300: periodic grids under 0.8 M nodes (1.2 M with a force field, and
- * where WARP does not apply; not where a thin grid fills its tiles badly, or is
- * long and fills less than 0.65 of them), walled ones under 1.25 M (1.5 x 2^20 where a side has fewer
- * than 256 nodes, 1.7 M with a force
- * field, any size where WARP does not apply).  Beyond that it picks WARP where
- * it applies, on a walled grid with the frame on the tile kernel (T2S2-FDLBM1),
- * and SCALAR otherwise; with path FUSED or a tile height given, WARP
- * where it applies, except on walled grids of fewer than 1.5 x 2^20 nodes, where
- * the frame launch's fixed cost makes the walls sweep faster, and SCALAR
- * otherwise.  T2S2-FDLBM2 takes WARP where it applies, except on walled grids of
- * fewer than 1.25 M nodes (1.5 x 2^20 where a side has fewer than 256 nodes).
+ * AUTO (with path AUTO and rows_per_cta 0) runs FP32 T2S2_1 grids of small and
+ * medium size on the tile kernel (one launch per step, a tile of 32 x 16 nodes
+ * per block through all stages in shared memory), where it is the fastest
+ * measured on GB300: periodic grids under 0.8 M nodes (1.2 M with a force field,
+ * and where WARP does not apply), but not those of many badly filled tiles, nor
+ * long thin ones that fill less than 0.65 of them; walled ones under 1.25 M (1.5
+ * x 2^20 where a side has fewer than 256 nodes, 1.7 M with a force field, any
+ * size where WARP does not apply).  Beyond that it picks WARP where it applies,
+ * on a walled grid with the frame on the tile kernel (on channels of few rows as
+ * the walls sweep), and SCALAR otherwise; with path FUSED or a tile height given,
+ * WARP where it applies, except on walled grids of fewer than 1.5 x 2^20 nodes,
+ * where the frame launch's fixed cost makes the walls sweep faster, and SCALAR
+ * otherwise.  T2S2_2 takes WARP where it applies, except on walled grids of fewer
+ * than 1.25 M nodes (1.5 x 2^20 where a side has fewer than 256 nodes).
  * Asking for a variant that does not apply returns FDLBM_EUNSUPPORTED; the
  * values 2 to 4 are not used. */
 enum { FDLBM_VARIANT_AUTO = 0, FDLBM_VARIANT_SCALAR = 1, FDLBM_VARIANT_WARP = 5 };
@@ -249,8 +249,8 @@ int fdlbm_kernels_per_step(fdlbm_t h);   /* kernel launches fdlbm_step makes per
  * The interior covers the nodes at least 4 from every wall whose tiles load
  * nothing outside the grid (Eq. 3.10 and the central differences next to a
  * wall reach no further), the frame the rest (with variant AUTO the frame of a
- * T2S2_1 grid runs on the tiles of the tile kernel instead, which store the
- * same nodes).  Host only, no device work:
+ * T2S2_1 grid, but for channels of few rows, runs on the tiles of the tile
+ * kernel instead, which store the same nodes).  Host only, no device work:
  * *count receives the number of tiles and at most cap are written to tiles.
  * EINVAL for bad arguments, EUNSUPPORTED where the warp-tile kernel does not
  * apply. */

@@ -10,13 +10,14 @@
 //       and the force cotangent, added in FP64
 //
 // The node maps are polynomials of second degree in the lattice velocity, so
-// their VJPs need only the lattice moments of the incoming cotangents (six, nine
+// their VJPs need only the lattice moments of the incoming cotangents (six, eight
 // with the forcing term of Eq. 3.12): no per-population derivative is formed.
 //
 // What bounds it: latency at two blocks per SM (98 KB of shared memory, 124
-// registers): issue slots 34 % busy, waits for global loads first; so the loads
-// of stage C' (g, the rest population of lam', the FP64 force gradient) are
-// issued before the barrier that precedes it (2048^2 274 -> 252 us), and the
+// registers): shared-memory pipe 65 %, issue slots 42 % busy, waits for global
+// loads and for dependent arithmetic first; so the loads of stage C' (g, the rest
+// population of lam', the FP64 force gradient) are issued before the barrier that
+// precedes it (2048^2 274 -> 252 us), and the
 // metrics before the previous step's results are needed.  Persistent blocks that
 // copied the next tile during stage C' were slower (278 us: 76 small copies per
 // thread and tile).  Against the sweep of adjoint.cu, which walks a chain of

@@ -627,7 +627,7 @@ fdlbm_status fdlbm_batch_create(int ncases, const fdlbm_grid *grids, const fdlbm
     if (b->precision == FDLBM_FP32_DEV) {
         for (fdlbm_ctx *h : b->cases) {
             // the case's own choice (its options, or the automatic one of a
-            // single grid, which leaves small walled grids to the walls sweep)
+            // single grid, which leaves small walled grids to the tile kernel)
             const bool want = h->variant == FDLBM_VARIANT_WARP;
             h->variant = FDLBM_VARIANT_SCALAR;
             if (!want || h->scheme != FDLBM_SCHEME_T2S2_1 ||

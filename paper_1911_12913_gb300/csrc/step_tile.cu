@@ -18,8 +18,8 @@
 // the domain, select the central one.  Outside a walled domain, loads read the
 // nearest node; no stored value depends on those.
 //
-// What bounds it: at 1024^2 (27 us per step, 39 GLUPS) the shared-memory pipe,
-// about 65 % busy with 38 64-bit loads per pair and stage; issue slots 43 % busy.
+// What bounds it: at 1025^2 (cavity, 29 us per step, 36 GLUPS) the shared-memory
+// pipe, 60 % busy with 38 64-bit loads per pair and stage; issue slots 42 % busy.
 // The tile's halo costs 1.9 times stage A and 1.4 times stage B.  On small grids
 // it is one tile's latency: 64^2 3.5 us per step, 257^2 cavity 4.9 (walls sweep
 // 9.8).  Tried: two rows per thread (tile 32 x 32, 128 registers) 2048^2 122 us
